@@ -116,7 +116,7 @@ struct gp_handle_s {
     bool scale_pending = false;
     long long step = 0;
     double t = 0;
-    int threads[3] = {64, 64, 64};
+    int threads[3] = {0, 0, 0};  // threads per block set by the caller or the autotuner; 0: default_threads
     bool contiguous_z = true;  // warp-tiled kernel for the stride-1 axis
     bool tma_z = true;         // ... through TMA tiles where the grid allows it
     int tma_lines = -1;        // axes (bit 0: x, bit 1: y) whose sweeps read through TMA boxes where the grid
@@ -432,6 +432,13 @@ int lines_per_thread(gp_handle h, int ax, int window) {
     return 1;
 }
 
+// Threads per block of the per-thread line solves.  64 for the windowed
+// forms (measured best of 64 and 128); 32 for the exact two-pass form: one
+// thread holds a whole line, so a grid of a few hundred warps is spread over
+// the SMs in units of one warp (240x200x160 x lines: 1000 warps are at most
+// 7 on an SM, in pairs 8).
+int default_threads(int window) { return window == 0 ? 32 : 64; }
+
 // Segments of one axis (see choose_segments).
 void segments(gp_handle h, int ax, int window, int *seg_len, int *n_seg) {
     choose_segments(geom(h), ax, window, lines_per_thread(h, ax, window), (int)h->elem, h->contiguous_z,
@@ -475,7 +482,7 @@ gp_status run_stage(gp_handle h, int stage, bool realtime) {
     const int mode = realtime ? 1 : 0;
     const int ax = stage;
     L.window = h->window[mode][ax];
-    L.threads = h->threads[ax];
+    L.threads = h->threads[ax] ? h->threads[ax] : default_threads(L.window);
     L.lpt = lines_per_thread(h, ax, L.window);
     L.contiguous = (ax == 2 && h->contiguous_z && L.window > 0) ? 1 : 0;
     int seg_len = 0, n_seg = 0;
@@ -1289,9 +1296,10 @@ gp_status autotune(gp_handle h, int realtime, int reps, const char *cache_path) 
         const int n = h->n[ax] - 2;
         std::vector<TuneChoice> cands;
         const int segs[] = {0, 64, 128, 256, n};
-        for (int th : {64, 128})
+        for (int th : {32, 64, 128})
             for (int sg : segs)
                 for (int lp : {4, 2, 1}) {
+                    if (th == 32 && h->window[mode][ax] != 0) continue;  // one-warp blocks: the exact form only
                     if (ax == 2 && lp != 1) continue;  // line groups apply to the strided axes only
                     if (ax < 2 && lp == 1 && fp16(h)) continue;  // FP16 storage moves two or four lines
                     if (h->window[mode][ax] == 0 && sg != 0) continue;  // the exact solve has no segments

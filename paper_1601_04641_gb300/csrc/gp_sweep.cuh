@@ -79,7 +79,11 @@ __device__ __forceinline__ void g_sincos(double x, double *s, double *c) { sinco
 //         |y| <= 0.05 (next term below 2^-27 of exp(-y)).
 //   FP64: sin through x^9, cos through x^10 for |x| <= 0.1 (next terms below
 //         2^-58 relative); exp(-y) - 1 through y^7 for |y| <= 0.02 (next
-//         term below 2^-60 of exp(-y)).
+//         term below 2^-60 of exp(-y)).  Groups of phases within 0.03 (the
+//         phases of a real-time step at dt = 0.02 d^2) take sin through x^7
+//         and cos through x^6 (next terms below 2^-58 and 2^-55): the FP64
+//         forms are bound by the FP64 pipe (2 lanes a clock and SM), and
+//         this saves 3 of the kick's operations.
 // Imaginary-time factors are formed as deviations from one (exp(-y) - 1,
 // and the trap tables hold exp(-dt V_a) - 1): a factor rounded once near one
 // and applied at every step acts as a potential error of u / dt (u the unit
@@ -88,7 +92,7 @@ __device__ __forceinline__ void g_sincos(double x, double *s, double *c) { sinco
 // rounded once is off by u |dt V|, a potential error of u |V|.
 template <typename R> struct Series;
 template <> struct Series<float> {
-    static constexpr float kTrig = 0.2f, kExp = 0.05f;
+    static constexpr float kTrig = 0.2f, kExp = 0.05f, kTrigNear = 0.f;  // no nearer tier
     __device__ __forceinline__ static void sincos(float x, float *sn, float *cs) {
         const float x2 = x * x;
         *sn = x * fmaf(x2, fmaf(x2, 1.f / 120.f, -1.f / 6.f), 1.f);
@@ -99,7 +103,12 @@ template <> struct Series<float> {
     }
 };
 template <> struct Series<double> {
-    static constexpr double kTrig = 0.1, kExp = 0.02;
+    static constexpr double kTrig = 0.1, kExp = 0.02, kTrigNear = 0.03;
+    __device__ __forceinline__ static void sincos_near(double x, double *sn, double *cs) {  // |x| <= kTrigNear
+        const double x2 = x * x;
+        *sn = x * fma(x2, fma(x2, fma(x2, -1.0 / 5040.0, 1.0 / 120.0), -1.0 / 6.0), 1.0);
+        *cs = fma(x2, fma(x2, fma(x2, -1.0 / 720.0, 1.0 / 24.0), -0.5), 1.0);
+    }
     __device__ __forceinline__ static void sincos(double x, double *sn, double *cs) {
         const double x2 = x * x;
         *sn = x * fma(x2, fma(x2, fma(x2, fma(x2, 1.0 / 362880.0, -1.0 / 5040.0), 1.0 / 120.0),
@@ -140,6 +149,19 @@ template <typename R> __device__ __forceinline__ R kick_expm1m(R y) {
 template <typename R> __device__ __forceinline__ R kick_dev(R ex, R eyz, R m) {
     const R t = fma(ex, eyz, ex + eyz);
     return fma(t, m, t + m);
+}
+
+// q (1 + ex)(1 + eyz)(1 + m).  FP64 applies the three deviations one after
+// the other: three operations on the FP64 pipe instead of five, each rounded
+// at the unit roundoff of the value.
+template <typename R> __device__ __forceinline__ R kick_apply(R q, R ex, R eyz, R m) {
+    if constexpr (sizeof(R) == 8) {
+        q = fma(q, ex, q);
+        q = fma(q, eyz, q);
+        return fma(q, m, q);
+    } else {
+        return fma(q, kick_dev(ex, eyz, m), q);
+    }
 }
 
 // Per-site kick state of one x line.  Imaginary time: exp(-dt V) is the
@@ -208,11 +230,16 @@ template <typename R> struct FImagReal : LineForm<R> {
         const V u = fma(k, dprev, r);
         return fma(u, ipm1, u);
     }
+    // FP64: fwd with c ip = -cp applied to dprev, one operation on the recurrence's chain instead of two
+    __device__ __forceinline__ static V fwd_chain(V r, V dprev, R k, C ipm1, C cp) {
+        if constexpr (sizeof(R) == 8) return fma(-cp, dprev, fma(r, ipm1, r));
+        else return fwd(r, dprev, k, ipm1);
+    }
     __device__ __forceinline__ static V back(V dp, C cp, V phi) { return fma(-cp, phi, dp); }
     __device__ __forceinline__ static R abs2(V v) { return v * v; }
     __device__ __forceinline__ static V kick(V p, const KickState<R> &k, int node) {
         const V q = p * k.s;
-        return fma(q, kick_dev(__ldg(k.ex + node), k.eyz, kick_expm1m(k.dtg * (q * q))), q);
+        return kick_apply(q, __ldg(k.ex + node), k.eyz, kick_expm1m(k.dtg * (q * q)));
     }
     // kick of NB consecutive nodes from node0: table loads issued together,
     // one series-range test per group, values equal kick's
@@ -233,7 +260,7 @@ template <typename R> struct FImagReal : LineForm<R> {
             }
             if (small) {
 #pragma unroll
-                for (int i = 0; i < G; ++i) v[g0 + i] = fma(q[i], kick_dev(ex[i], k.eyz, Series<R>::expm1m(y[i])), q[i]);
+                for (int i = 0; i < G; ++i) v[g0 + i] = kick_apply(q[i], ex[i], k.eyz, Series<R>::expm1m(y[i]));
             } else {
 #pragma unroll
                 for (int i = 0; i < G; ++i) v[g0 + i] = kick(v[g0 + i], k, node0 + g0 + i);
@@ -255,6 +282,11 @@ template <typename R> struct FImagCplx : LineForm<cx<R>> {
     __device__ __forceinline__ static V fwd(V r, V dprev, R k, C ipm1) {
         const R ure = fma(k, dprev.re, r.re), uim = fma(k, dprev.im, r.im);
         return V{fma(ure, ipm1, ure), fma(uim, ipm1, uim)};
+    }
+    __device__ __forceinline__ static V fwd_chain(V r, V dprev, R k, C ipm1, C cp) {
+        if constexpr (sizeof(R) == 8)
+            return V{fma(-cp, dprev.re, fma(r.re, ipm1, r.re)), fma(-cp, dprev.im, fma(r.im, ipm1, r.im))};
+        else return fwd(r, dprev, k, ipm1);
     }
     __device__ __forceinline__ static V back(V dp, C cp, V phi) {
         return V{fma(-cp, phi.re, dp.re), fma(-cp, phi.im, dp.im)};
@@ -313,11 +345,17 @@ template <typename R> struct FRealTime : LineForm<cx<R>> {
         const R uim = fma(k, dprev.re, r.im);
         return V{fma(ure, ipm1.re, fma(-uim, ipm1.im, ure)), fma(ure, ipm1.im, fma(uim, ipm1.re, uim))};
     }
+    // (-cp is complex: four products on dprev instead of two, so fwd's two are fewer operations)
+    __device__ __forceinline__ static V fwd_chain(V r, V dprev, R k, C ipm1, C) { return fwd(r, dprev, k, ipm1); }
     __device__ __forceinline__ static V back(V dp, C cp, V phi) {
         // dp - cp * phi
-        R pre = fma(cp.re, phi.re, -cp.im * phi.im);
-        R pim = fma(cp.re, phi.im, cp.im * phi.re);
-        return V{dp.re - pre, dp.im - pim};
+        if constexpr (sizeof(R) == 8) {  // four operations on the FP64 pipe instead of six
+            return V{fma(-cp.re, phi.re, fma(cp.im, phi.im, dp.re)), fma(-cp.re, phi.im, fma(-cp.im, phi.re, dp.im))};
+        } else {
+            R pre = fma(cp.re, phi.re, -cp.im * phi.im);
+            R pim = fma(cp.re, phi.im, cp.im * phi.re);
+            return V{dp.re - pre, dp.im - pim};
+        }
     }
     __device__ __forceinline__ static R abs2(V v) { return fma(v.re, v.re, v.im * v.im); }
     __device__ __forceinline__ static V kick(V p, const KickState<R> &k, int node) {
@@ -335,14 +373,31 @@ template <typename R> struct FRealTime : LineForm<cx<R>> {
             constexpr int G = NB < kKickGroup ? NB : kKickGroup;
             R px[G], th[G];
             V q[G];
-            bool small = true;
+            bool small = true, near = Series<R>::kTrigNear > R(0);
 #pragma unroll
             for (int i = 0; i < G; ++i) px[i] = __ldg(k.px + node0 + g0 + i);
 #pragma unroll
+            for (int i = 0; i < G; ++i) q[i] = v[g0 + i];
+            if (sizeof(R) == 4 || k.s != R(1)) {  // FP64: no product where nothing is pending (s is one value per launch)
+#pragma unroll
+                for (int i = 0; i < G; ++i) q[i] = V{q[i].re * k.s, q[i].im * k.s};
+            }
+#pragma unroll
             for (int i = 0; i < G; ++i) {
-                q[i] = V{v[g0 + i].re * k.s, v[g0 + i].im * k.s};
                 th[i] = fma(k.dtg, abs2(q[i]), px[i] + k.pyz);
                 small = small && fabs(th[i]) <= Series<R>::kTrig;
+                near = near && fabs(th[i]) <= Series<R>::kTrigNear;
+            }
+            if constexpr (sizeof(R) == 8) {
+                if (near) {
+#pragma unroll
+                    for (int i = 0; i < G; ++i) {
+                        R sn, cs;
+                        Series<R>::sincos_near(th[i], &sn, &cs);
+                        v[g0 + i] = V{fma(cs, q[i].re, sn * q[i].im), fma(cs, q[i].im, -sn * q[i].re)};
+                    }
+                    continue;
+                }
             }
             if (small) {
 #pragma unroll
@@ -377,6 +432,9 @@ template <class F> struct FPair {
     }
     __device__ __forceinline__ static V fwd(V r, V dprev, Real k, C ipm1) {
         return V{F::fwd(r.a, dprev.a, k, ipm1), F::fwd(r.b, dprev.b, k, ipm1)};
+    }
+    __device__ __forceinline__ static V fwd_chain(V r, V dprev, Real k, C ipm1, C cp) {
+        return V{F::fwd_chain(r.a, dprev.a, k, ipm1, cp), F::fwd_chain(r.b, dprev.b, k, ipm1, cp)};
     }
     __device__ __forceinline__ static V back(V dp, C cp, V phi) {
         return V{F::back(dp.a, cp, phi.a), F::back(dp.b, cp, phi.b)};
@@ -445,6 +503,7 @@ struct PRealTimeF {
         const float2 pim = fma2(dup2(cp.re), phi.im, mul2(dup2(cp.im), phi.re));
         return V{sub2(dp.re, pre), sub2(dp.im, pim)};
     }
+    __device__ __forceinline__ static V fwd_chain(V r, V dprev, float k, C ipm1, C) { return fwd(r, dprev, k, ipm1); }
     __device__ __forceinline__ static float abs2(V v) {
         const float2 s = fma2(v.re, v.re, mul2(v.im, v.im));
         return s.x + s.y;
@@ -544,6 +603,7 @@ struct PImagRealF {
         const float2 u = fma2(dup2(k), dprev, r);
         return fma2(u, dup2(ipm1), u);
     }
+    __device__ __forceinline__ static V fwd_chain(V r, V dprev, float k, C ipm1, C) { return fwd(r, dprev, k, ipm1); }
     __device__ __forceinline__ static V back(V dp, C cp, V phi) { return fma2(dup2(-cp), phi, dp); }
     __device__ __forceinline__ static float abs2(V v) {
         const float2 s = mul2(v, v);
@@ -621,6 +681,7 @@ struct PImagCplxF {
     __device__ __forceinline__ static V fwd(V r, V dprev, float k, C ipm1) {
         return V{PImagRealF::fwd(r.re, dprev.re, k, ipm1), PImagRealF::fwd(r.im, dprev.im, k, ipm1)};
     }
+    __device__ __forceinline__ static V fwd_chain(V r, V dprev, float k, C ipm1, C) { return fwd(r, dprev, k, ipm1); }
     __device__ __forceinline__ static V back(V dp, C cp, V phi) {
         return V{PImagRealF::back(dp.re, cp, phi.re), PImagRealF::back(dp.im, cp, phi.im)};
     }
@@ -988,27 +1049,81 @@ __device__ __forceinline__ void solve_segment(int n, int tb, int te, int tconst,
 }
 
 // Exact two-pass Thomas over a whole line (window 0): dp is staged in the
-// output and read back by the backward sweep.  Direct loads and stores.
+// output and read back by the backward sweep.  Both passes go in chunks of
+// kExactChunk nodes with the next chunk's loads issued before the current
+// one's arithmetic: a node loaded, kicked and used in one iteration kept
+// every node waiting for its load and its kick (64x48x40 FP64 real, kick + x
+// 124 us a launch; 240x200x160 FP64 complex 738 us).  Chunks whose
+// coefficients have settled take them from registers.
+constexpr int kExactChunk = 8;
 template <class F, typename R, class IO>
-__device__ __forceinline__ void solve_line_exact(int n, R kap, const typename F::C *__restrict__ cp,
+__device__ __forceinline__ void solve_line_exact(int n, int tconst, R kap, const typename F::C *__restrict__ cp,
                                                  const typename F::C *__restrict__ ipm1, IO &io) {
     using V = typename F::V;
-    V pm = F::zero();
-    V p0 = io.load1(0);
-    V p1 = io.load1(1);
-    V dprev = F::zero();
-    for (int t = 0; t < n; ++t) {
-        dprev = F::fwd(F::rhs(pm, p0, p1, kap), dprev, kap, ldc(ipm1 + t));
-        pm = p0;
-        p0 = p1;
-        p1 = io.load1(t + 2);
-        if (t < n - 1) io.stage(t, dprev);
+    using C = typename F::C;
+    constexpr int CH = kExactChunk;
+    const C cps = ldc(cp + n - 1), ips = ldc(ipm1 + n - 1);
+    V pm = F::zero(), p0 = F::zero(), dprev = F::zero();
+    V nxt[CH], cur[CH];
+    io.load_chunk(0, nxt);
+    for (int t0 = 0; t0 <= n; t0 += CH) {  // positions t0 .. t0+CH-1 give dp[t0-1 .. t0+CH-2]
+#pragma unroll
+        for (int q = 0; q < CH; ++q) cur[q] = nxt[q];
+        if (t0 + CH <= n) io.load_chunk(t0 + CH, nxt);
+        io.kick_chunk(t0, cur);
+        auto full = [&](auto settled) {
+            constexpr bool S = decltype(settled)::value;
+#pragma unroll
+            for (int q = 0; q < CH; ++q) {
+                const int t = t0 + q - 1;
+                dprev = F::fwd_chain(F::rhs(pm, p0, cur[q], kap), dprev, kap, S ? ips : ldc(ipm1 + t), S ? cps : ldc(cp + t));
+                io.stage(t, dprev);
+                pm = p0;
+                p0 = cur[q];
+            }
+        };
+        if (t0 > 0 && t0 + CH <= n + 1) {
+            if (t0 - 1 >= tconst) full(std::true_type{});
+            else full(std::false_type{});
+        } else {
+#pragma unroll
+            for (int q = 0; q < CH; ++q) {
+                const int t = t0 + q - 1;
+                if (t >= 0 && t < n) {
+                    dprev = F::fwd_chain(F::rhs(pm, p0, cur[q], kap), dprev, kap, ldc(ipm1 + t), ldc(cp + t));
+                    io.stage(t, dprev);
+                }
+                pm = p0;
+                p0 = cur[q];
+            }
+        }
     }
     V phi = dprev;
     io.put1(n - 1, phi);
-    for (int t = n - 2; t >= 0; --t) {
-        phi = F::back(io.unstage(t), ldc(cp + t), phi);
-        io.put1(t, phi);
+    auto unstage = [&](int t) {  // dp[t], dp[t-1], ...
+#pragma unroll
+        for (int q = 0; q < CH; ++q)
+            if (t - q >= 0) nxt[q] = io.unstage(t - q);
+    };
+    unstage(n - 2);
+    for (int t0 = n - 2; t0 >= 0; t0 -= CH) {
+#pragma unroll
+        for (int q = 0; q < CH; ++q) cur[q] = nxt[q];
+        unstage(t0 - CH);
+        if (t0 - CH + 1 >= tconst) {
+#pragma unroll
+            for (int q = 0; q < CH; ++q) {
+                phi = F::back(cur[q], cps, phi);
+                io.put1(t0 - q, phi);
+            }
+        } else {
+#pragma unroll
+            for (int q = 0; q < CH; ++q)
+                if (t0 - q >= 0) {
+                    phi = F::back(cur[q], ldc(cp + t0 - q), phi);
+                    io.put1(t0 - q, phi);
+                }
+        }
     }
 }
 
@@ -1085,9 +1200,28 @@ template <class F, class M, typename R, int KIND> struct DirectIO {
     long long st;
     int n;
     Hooks<F, M, R, KIND> hk;
-    __device__ __forceinline__ V load1(int t) const {
-        if (t < 0 || t >= n) return M::zero();
-        return hk.on_load(t, M::load(in[(long long)(t + 1) * st]));
+    // values at positions p .. p+NB-1 as stored, zeros from n on
+    template <int NB> __device__ __forceinline__ void load_chunk(int p, V (&v)[NB]) const {
+        const MV *g = in + (long long)(p + 1) * st;
+        if (p + NB <= n) {
+#pragma unroll
+            for (int q = 0; q < NB; ++q) v[q] = M::load(g[q * st]);
+        } else {
+#pragma unroll
+            for (int q = 0; q < NB; ++q) v[q] = p + q < n ? M::load(g[q * st]) : M::zero();
+        }
+    }
+    // the kick of positions p .. p+NB-1 (those from n on stay zero)
+    template <int NB> __device__ __forceinline__ void kick_chunk(int p, V (&v)[NB]) const {
+        if constexpr (KIND == K_X) {
+            if (p + NB <= n) {
+                hk.on_load_chunk(p, v);
+            } else {
+#pragma unroll
+                for (int q = 0; q < NB; ++q)
+                    if (p + q < n) v[q] = hk.on_load(p + q, v[q]);
+            }
+        }
     }
     __device__ __forceinline__ void put1(int t, V v) const {
         out[(long long)(t + 1) * st] = M::store(v);
@@ -1211,7 +1345,7 @@ __device__ __forceinline__ double lines_body(const SweepArgs &a, unsigned bx, un
             io.n = n;
             io.hk.acc = &acc;
             io.hk.init(a, L);
-            solve_line_exact<M, R>(n, (R)a.kappa, cp, ipm1, io);
+            solve_line_exact<M, R>(n, a.t_const, (R)a.kappa, cp, ipm1, io);
         }
     }
     return acc.value();
