@@ -108,6 +108,7 @@ struct gp_handle_s {
     Tables tab;                         // offsets of the coefficient tables in d_coef
     int window[2][3] = {{0, 0, 0}, {0, 0, 0}};  // window in use per mode and axis
     int forced_window = -1;
+    bool axis_window[3] = {false, false, false};  // a window set for this axis alone (gp_set_axis_window)
     double *d_scal = nullptr;
     double *d_obs = nullptr;
     double *d_partials = nullptr;
@@ -217,7 +218,7 @@ Geometry geom(gp_handle h) {
 gp_status build_coefficients(gp_handle h) {
     const bool f32 = h->prec != GP_F64;  // FP32 tables for FP32 arithmetic (FP32 and FP16 storage)
     std::vector<char> host;
-    append_tables(geom(h), f32, modes_of(h), host, h->tab);
+    append_tables(geom(h), f32, modes_of(h), host, h->tab, kPcrChosen);
     const size_t off = host.size();
     for (int mode = 0; mode < modes_of(h); ++mode)
         for (int ax = 0; ax < 3; ++ax) {
@@ -228,6 +229,7 @@ gp_status build_coefficients(gp_handle h) {
                 w = h->forced_window;
             h->window[mode][ax] = w;
         }
+    for (bool &set : h->axis_window) set = false;
     if (h->d_coef && h->coef_bytes < off) {
         cudaFree(h->d_coef);
         h->d_coef = nullptr;
@@ -426,6 +428,9 @@ gp_status check_status(gp_handle h) {
 // a windowed solve (the form that has a four-line variant).
 int lines_per_thread(gp_handle h, int ax, int window) {
     if (ax == 2 || h->elem > 8) return 1;
+    // FP64 exact solves are bound by the FP64 pipe, which a pair does not
+    // relieve: one line a thread, for twice the warps (unless set)
+    if (h->prec == GP_F64 && window == 0 && h->max_lpt[ax] == 4) return 1;
     auto fits = [&](int g) { return sweep_lines(h, ax) % g == 0 && (ax != 1 || h->n[2] % g == 0); };
     if (h->max_lpt[ax] >= 4 && (h->elem == 4 || h->elem == 2) && window > 0 && fits(4)) return 4;  // real fields
     if (h->max_lpt[ax] >= 2 && fits(2)) return 2;
@@ -436,8 +441,9 @@ int lines_per_thread(gp_handle h, int ax, int window) {
 // forms (measured best of 64 and 128); 32 for the exact two-pass form: one
 // thread holds a whole line, so a grid of a few hundred warps is spread over
 // the SMs in units of one warp (240x200x160 x lines: 1000 warps are at most
-// 7 on an SM, in pairs 8).
-int default_threads(int window) { return window == 0 ? 32 : 64; }
+// 7 on an SM, in pairs 8).  The z sweep keeps 64: its blocks are the norm's
+// partial sums, which the batched launch groups the same way.
+int default_threads(int ax, int window) { return window == 0 && ax < 2 ? 32 : 64; }
 
 // Segments of one axis (see choose_segments).
 void segments(gp_handle h, int ax, int window, int *seg_len, int *n_seg) {
@@ -482,7 +488,7 @@ gp_status run_stage(gp_handle h, int stage, bool realtime) {
     const int mode = realtime ? 1 : 0;
     const int ax = stage;
     L.window = h->window[mode][ax];
-    L.threads = h->threads[ax] ? h->threads[ax] : default_threads(L.window);
+    L.threads = h->threads[ax] ? h->threads[ax] : default_threads(ax, L.window);
     L.lpt = lines_per_thread(h, ax, L.window);
     L.contiguous = (ax == 2 && h->contiguous_z && L.window > 0) ? 1 : 0;
     int seg_len = 0, n_seg = 0;
@@ -515,7 +521,21 @@ gp_status run_stage(gp_handle h, int stage, bool realtime) {
     const int zthreads = L.contiguous ? 32 : L.threads;
     if (stage == 2 && blocks_for(a.n_lines, zthreads) * (size_t)a.n_seg > h->partial_cap)
         return fail(h, GP_ERR_STATE, "z sweep grid exceeds the partials buffer");
-    GP_CK(h, launch_sweep(L, a, h->stream));
+    // FP64 at its automatic settings: by cyclic reduction where the lines are
+    // too few to fill the GPU one thread each (a window, a segment length or
+    // a block size that the caller set keeps the per-thread solve)
+    PcrArgs pcr;
+    const AxisTables &at = h->tab.ax[mode][ax];
+    if (h->prec == GP_F64 && L.window == 0 && h->forced_window < 0 && !h->axis_window[ax] && h->threads[ax] == 0 &&
+        h->seg_override[ax] == 0 && choose_pcr(a.n_lines, a.N - 2, L.form, L.kind, at.pcr_levels, (int)h->elem, &pcr.tl) &&
+        blocks_for(a.n_lines, pcr.tl) <= h->partial_cap) {
+        pcr.levels = at.pcr_levels;
+        pcr.lv = h->d_coef + at.off_pcr;
+        pcr.im1 = h->d_coef + at.off_pcr_inv;
+        GP_CK(h, launch_sweep_pcr(L.form, L.kind, a, pcr, h->stream));
+    } else {
+        GP_CK(h, launch_sweep(L, a, h->stream));
+    }
     h->cur ^= 1;
     if (stage == 0) h->scale_pending = false;
     if (stage == 2 && !realtime) h->scale_pending = true;
@@ -1061,6 +1081,7 @@ gp_status gp_set_window(gp_handle h, int window) {
         for (int ax = 0; ax < 3; ++ax)
             h->window[mode][ax] = window >= 0 ? window : default_window(h->tab.ax[mode][ax], h->prec != GP_F64);
     h->forced_window = window;
+    for (bool &set : h->axis_window) set = false;
     drop_graphs(h);
     return GP_OK;
 }
@@ -1077,6 +1098,7 @@ gp_status gp_set_axis_window(gp_handle h, int axis, int window) {
         if (h->n[axis] > 1 && window > 0 && (at.min_window == 0 || window < at.min_window))
             return fail(h, GP_ERR_ARG, "window too small for the accuracy of this dt");
     }
+    h->axis_window[axis] = window >= 0;
     for (int mode = 0; mode < modes_of(h); ++mode)
         h->window[mode][axis] = window >= 0 ? window : default_window(h->tab.ax[mode][axis], h->prec != GP_F64);
     drop_graphs(h);
@@ -1296,10 +1318,10 @@ gp_status autotune(gp_handle h, int realtime, int reps, const char *cache_path) 
         const int n = h->n[ax] - 2;
         std::vector<TuneChoice> cands;
         const int segs[] = {0, 64, 128, 256, n};
-        for (int th : {32, 64, 128})
+        for (int th : {0, 32, 64, 128})  // 0: the automatic choice
             for (int sg : segs)
                 for (int lp : {4, 2, 1}) {
-                    if (th == 32 && h->window[mode][ax] != 0) continue;  // one-warp blocks: the exact form only
+                    if (th <= 32 && h->window[mode][ax] != 0) continue;  // the exact (FP64) form only
                     if (ax == 2 && lp != 1) continue;  // line groups apply to the strided axes only
                     if (ax < 2 && lp == 1 && fp16(h)) continue;  // FP16 storage moves two or four lines
                     if (h->window[mode][ax] == 0 && sg != 0) continue;  // the exact solve has no segments

@@ -12,9 +12,15 @@
 // -- then the z line solves through the Cartesian z-sweep kernels, and in
 // imaginary time the renormalisation in the cylindrical measure
 // 2 pi rho drho dz (a weighted norm reduction; the factor is applied by
-// the next kick).  The radial kernel runs one thread per z line (threads
-// of a warp own adjacent z, so each node's load and store is one
-// contiguous row) with the exact two-pass Thomas algorithm.
+// the next kick).
+//
+// These grids are small (120x241: 28 k sites), so every part of a step is
+// spread over the whole GPU.  FP64: both sweeps by truncated cyclic reduction
+// (gp_pcr.cuh), the z sweep carrying the weighted norm, two launches a step.
+// FP32: the radial Thomas recurrences run on lines held in shared memory, a
+// few lines a block, with the kick and the right-hand side spread over the
+// block; then the z sweep and a norm reduction.  Lines too long for shared
+// memory take one thread per z line with values staged in global memory.
 #include "gp.h"
 #include "gp_host.h"
 #include "gp_internal.h"
@@ -141,88 +147,184 @@ __global__ void __launch_bounds__(128) axial_radial_kernel(AxArgs a) {
     }
 }
 
-// Sums over the grid in the cylindrical measure, FP64: per-block partials of
-// NV quantities, then one block adds them in block order (deterministic).
-constexpr int kRedThreads = 256;
-constexpr int kRedBlocks = 304;
-
-__device__ __forceinline__ double ax_block_sum(double v) {
-    __shared__ double red[kRedThreads / 32];
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+// Kick and radial CN solve of tl adjacent z lines per block, held in shared
+// memory: the kick and the right-hand side run over all (node, line) pairs
+// of the block, the two recurrences one thread per line in chunks whose loads
+// come first.  The arithmetic is axial_radial_kernel's.
+constexpr int kRadialThreads = 128;
+constexpr int kRadialChunk = 8;
+template <typename R, bool CPLX>
+__global__ void __launch_bounds__(kRadialThreads) axial_radial_smem_kernel(AxArgs a, int tl) {
+    using E = AxElem<R, CPLX>;
+    using V = typename E::V;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int n = a.nx - 2, k0 = blockIdx.x * tl, nl = min(tl, a.nz - k0), total = n * nl;
+    V *x = reinterpret_cast<V *>(smem_raw), *y = x + (size_t)n * tl;
+    const V *in = static_cast<const V *>(a.in);
+    V *out = static_cast<V *>(a.out);
+    const Cx<R> *A = static_cast<const Cx<R> *>(a.A), *C = static_cast<const Cx<R> *>(a.C);
+    const Cx<R> *cp = static_cast<const Cx<R> *>(a.cp), *ip = static_cast<const Cx<R> *>(a.ip);
+    const long long nz = a.nz;
+    const R sc = (R)__ldg(a.scale);
+    for (int s = threadIdx.x; s < total; s += kRadialThreads) {
+        const int t = s / nl, k = k0 + s - t * nl;
+        V v = E::zero();  // the z boundary: zero whatever the input holds
+        if (k > 0 && k < a.nz - 1) {
+            const double z = a.z0 + k * a.dz, vz = 0.5 * a.lambda2 * z * z;
+            v = ax_kick<R, CPLX>(a, in[(t + 1) * nz + k], sc, t + 1, vz);
+        }
+        x[s] = v;
+    }
+    for (int q = threadIdx.x; q < 2 * nl; q += kRadialThreads) out[(q < nl ? 0 : (a.nx - 1) * nz - nl) + k0 + q] = E::zero();
     __syncthreads();
-    if (lane == 0) red[wid] = v;
+    for (int s = threadIdx.x; s < total; s += kRadialThreads) {
+        const int t = s / nl;
+        const V pm = t > 0 ? x[s - nl] : E::zero(), p0 = x[s], p1 = t < n - 1 ? x[s + nl] : E::zero();
+        y[s] = E::add(p0, E::add(E::mul(A[t], E::sub(pm, p0)), E::mul(C[t], E::sub(p1, p0))));
+    }
     __syncthreads();
-    double t = 0.0;
-    if (threadIdx.x == 0)
-        for (int w = 0; w < kRedThreads / 32; ++w) t += red[w];
-    return t;
+    if ((int)threadIdx.x < nl) {
+        V *col = y + threadIdx.x;
+        V dp = E::zero();
+        for (int t0 = 0; t0 < n; t0 += kRadialChunk) {
+            V r[kRadialChunk];
+            Cx<R> at[kRadialChunk], it[kRadialChunk];
+#pragma unroll
+            for (int q = 0; q < kRadialChunk; ++q) {
+                const int t = min(t0 + q, n - 1);
+                r[q] = col[t * nl];
+                at[q] = A[t];
+                it[q] = ip[t];
+            }
+#pragma unroll
+            for (int q = 0; q < kRadialChunk; ++q)
+                if (t0 + q < n) {
+                    dp = E::mul(it[q], E::add(r[q], E::mul(at[q], dp)));
+                    col[(t0 + q) * nl] = dp;
+                }
+        }
+        V phi = dp;
+        for (int t0 = n - 2; t0 >= 0; t0 -= kRadialChunk) {
+            V r[kRadialChunk];
+            Cx<R> ct[kRadialChunk];
+#pragma unroll
+            for (int q = 0; q < kRadialChunk; ++q) {
+                const int t = max(t0 - q, 0);
+                r[q] = col[t * nl];
+                ct[q] = cp[t];
+            }
+#pragma unroll
+            for (int q = 0; q < kRadialChunk; ++q)
+                if (t0 - q >= 0) {
+                    phi = E::sub(r[q], E::mul(ct[q], phi));
+                    col[(t0 - q) * nl] = phi;
+                }
+        }
+    }
+    __syncthreads();
+    for (int s = threadIdx.x; s < total; s += kRadialThreads) {
+        const int t = s / nl;
+        out[(t + 1) * nz + k0 + s - t * nl] = y[s];
+    }
 }
+
+// Sums over the grid in the cylindrical measure, FP64: per-block partials of
+// 6 quantities (or the first alone), added in block order by the last block
+// to finish (deterministic).  One site per thread on a 120x241 grid: the sums
+// are bound by the FP64 pipe, which works at 64 clocks per warp instruction
+// however few lanes are active, so the blocks are many and short.  (One block
+// adding 304 partials with one thread per quantity took 27 us, the sums with
+// a division per site 14 us; now 4 us together.)
+constexpr int kRedThreads = 192;  // one warp per quantity in the last block
+constexpr int kRedBlocks = 304;
 
 struct AxSums {
     const void *psi;
     int nx, nz;
-    double drho, dz, z0, gamma2, lambda2;
+    double drho, dz, z0, hg2, hl2;  // hg2, hl2: half the squared trap frequencies
+    double w0, kr, kz;              // 2 pi drho dz; the kinetic weights pi dz / drho and pi drho / dz
+    double g;
     const double *scale;  // applied to psi on read
     double *partials;     // kRedBlocks x 6
+    unsigned int *counter;
+    double *out;          // [0] norm, [1] mu, [2] E, [3] rms_x = rms_y, [4] rms_z, [5] finite flag (null: none)
+    double *scale_out;    // the renormalisation factor 1 / sqrt(norm) (null: none)
 };
 
 // Per-block sums (weight w = 2 pi rho_i drho dz): [0] w|psi|^2, [1] w V|psi|^2,
 // [2] w|psi|^4, [3] w rho^2|psi|^2, [4] w z^2|psi|^2, [5] the kinetic form
 // (radial links weighted 2 pi rho_{i+1/2} dz / drho, z links 2 pi rho_i drho / dz, times 1/2).
-template <typename R, bool CPLX>
+// NV = 1: the norm alone.
+template <typename R, bool CPLX, int NV>
 __global__ void __launch_bounds__(kRedThreads) axial_sums_kernel(AxSums a) {
     using E = AxElem<R, CPLX>;
     using V = typename E::V;
+    __shared__ double red[kRedThreads / 32][NV];
+    __shared__ double tot[NV];
+    __shared__ int is_last;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const V *psi = static_cast<const V *>(a.psi);
     const double s2 = (*a.scale) * (*a.scale);
     const long long sites = (long long)a.nx * a.nz;
-    double acc[6] = {0, 0, 0, 0, 0, 0};
-    const double two_pi = 6.283185307179586;
+    double acc[NV] = {};
     for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < sites;
          q += (long long)gridDim.x * blockDim.x) {
         const int i = (int)(q / a.nz), k = (int)(q % a.nz);
         if (i < 1 || i > a.nx - 2) continue;
         const V p = psi[q];
-        const double rho = E::abs2(p) * s2;
-        const double r = (i - 0.5) * a.drho, z = a.z0 + k * a.dz, w = two_pi * r * a.drho * a.dz;
-        acc[0] += w * rho;
-        acc[1] += w * 0.5 * (a.gamma2 * r * r + a.lambda2 * z * z) * rho;
-        acc[2] += w * rho * rho;
-        acc[3] += w * r * r * rho;
-        acc[4] += w * z * z * rho;
-        const double dr = E::abs2(E::sub(psi[q + a.nz], p)) * s2;  // link to node i + 1
-        double kin = 0.5 * two_pi * (r + 0.5 * a.drho) * a.dz / a.drho * dr;
-        if (k + 1 < a.nz) kin += 0.5 * two_pi * r * a.drho / a.dz * E::abs2(E::sub(psi[q + 1], p)) * s2;
-        acc[5] += kin;
+        const double r = (i - 0.5) * a.drho, rho = E::abs2(p) * s2, w = a.w0 * r, wr = w * rho;
+        acc[0] += wr;
+        if constexpr (NV > 1) {
+            const double z = a.z0 + k * a.dz, r2 = r * r, z2 = z * z;
+            acc[1] = fma(fma(a.hg2, r2, a.hl2 * z2), wr, acc[1]);
+            acc[2] = fma(wr, rho, acc[2]);
+            acc[3] = fma(r2, wr, acc[3]);
+            acc[4] = fma(z2, wr, acc[4]);
+            const double dr = E::abs2(E::sub(psi[q + a.nz], p)) * s2;  // link to node i + 1
+            double kin = a.kr * (r + 0.5 * a.drho) * dr;
+            if (k + 1 < a.nz) kin += a.kz * r * (E::abs2(E::sub(psi[q + 1], p)) * s2);
+            acc[5] += kin;
+        }
     }
-    for (int v = 0; v < 6; ++v) {
-        const double t = ax_block_sum(acc[v]);
-        if (threadIdx.x == 0) a.partials[blockIdx.x * 6 + v] = t;
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+        for (int o = 16; o > 0; o >>= 1) acc[v] += __shfl_xor_sync(0xffffffffu, acc[v], o);
+        if (lane == 0) red[wid][v] = acc[v];
     }
-}
-
-// out: [0] norm, [1] mu, [2] E, [3] rms_x = rms_y, [4] rms_z, [5] finite flag;
-// with scale_out: the renormalisation factor 1 / sqrt(norm).
-__global__ void axial_finish_kernel(const double *partials, int blocks, double g, double *out, double *scale_out) {
-    __shared__ double tot[6];
-    if (threadIdx.x < 6) {
+    __syncthreads();
+    if (threadIdx.x < NV) {
         double t = 0.0;
-        for (int b = 0; b < blocks; ++b) t += partials[b * 6 + threadIdx.x];
-        tot[threadIdx.x] = t;
+        for (int w = 0; w < kRedThreads / 32; ++w) t += red[w][threadIdx.x];
+        a.partials[blockIdx.x * NV + threadIdx.x] = t;
+        __threadfence();
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) is_last = atomicAdd(a.counter, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!is_last) return;
+    __threadfence();
+    if (wid < NV) {
+        double t = 0.0;
+        for (unsigned b = lane; b < gridDim.x; b += 32) t += __ldcg(a.partials + b * NV + wid);
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (lane == 0) tot[wid] = t;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
         const double nrm = tot[0];
-        out[0] = nrm;
-        out[1] = (tot[5] + tot[1] + g * tot[2]) / nrm;
-        out[2] = (tot[5] + tot[1] + 0.5 * g * tot[2]) / nrm;
-        out[3] = sqrt(0.5 * tot[3] / nrm);
-        out[4] = sqrt(tot[4] / nrm);
-        bool fin = true;
-        for (int q = 0; q < 5; ++q) fin = fin && isfinite(out[q]);
-        out[5] = fin ? 1.0 : 0.0;
-        if (scale_out) *scale_out = 1.0 / sqrt(nrm);
+        if constexpr (NV > 1) {
+            double *out = a.out;
+            out[0] = nrm;
+            out[1] = (tot[5] + tot[1] + a.g * tot[2]) / nrm;
+            out[2] = (tot[5] + tot[1] + 0.5 * a.g * tot[2]) / nrm;
+            out[3] = sqrt(0.5 * tot[3] / nrm);
+            out[4] = sqrt(tot[4] / nrm);
+            bool fin = true;
+            for (int q = 0; q < 5; ++q) fin = fin && isfinite(out[q]);
+            out[5] = fin ? 1.0 : 0.0;
+        }
+        if (a.scale_out) *a.scale_out = 1.0 / sqrt(nrm);
+        *a.counter = 0u;
     }
 }
 
@@ -270,6 +372,10 @@ struct gp_axial_s {
     char *d_tab = nullptr;
     Tables T;                  // Cartesian tables of the (nx, 1, nz) grid: the z sweep's
     size_t rad_off[2][4] = {};  // [mode][A, C, cp, ip] byte offsets in d_tab
+    int rad_levels[2] = {0, 0};  // FP64: cyclic-reduction levels of the radial matrix (0: no tables)
+    size_t rad_pcr[2][3] = {};   // [mode][level tables, final inverse, right-hand side]
+    size_t rad_kick = 0, rad_phase = 0;  // exp(-dt gamma^2 rho^2 / 2) - 1 and dt gamma^2 rho^2 / 2 per radial node
+    size_t line_w = 0;           // 2 pi rho_i drho dz per radial node, 0 on the ghost and the boundary
     double *d_scal = nullptr, *d_part = nullptr, *d_obs = nullptr;
     unsigned int *d_counter = nullptr;
     size_t part_cap = 0;
@@ -353,7 +459,63 @@ void append_radial(gp_axial a, int mode, std::vector<char> &host) {
     }
 }
 
+// FP64 tables of the cyclic-reduction form of a mode: the radial matrix's
+// reduction and its right-hand side's coefficients.
+void append_radial_pcr(gp_axial a, int mode, std::vector<char> &host) {
+    using Z = std::complex<double>;
+    const int n = a->nx - 2;
+    const double k = a->dt / (4.0 * a->drho * a->drho);
+    const Z c = mode == 1 ? Z(0.0, k) : Z(k, 0.0);
+    std::vector<Z> A(n), C(n), E(n);
+    for (int t = 0; t < n; ++t) {
+        const double r = t + 0.5;  // in units of drho
+        A[t] = c * ((r - 0.5) / r);
+        C[t] = c * ((r + 0.5) / r);
+        E[t] = A[t] + C[t];
+    }
+    a->rad_levels[mode] = append_pcr(host, A, E, C, mode == 1, &a->rad_pcr[mode][0], &a->rad_pcr[mode][1]);
+    const size_t esz = (mode == 1 ? 2 : 1) * sizeof(double), off = align_up(host.size(), 256);
+    a->rad_pcr[mode][2] = off;
+    host.resize(align_up(off + 2 * n * esz, 256), 0);
+    for (int t = 0; t < n; ++t)
+        for (int q = 0; q < 2; ++q) {
+            const Z v = q ? C[t] : A[t];
+            const double d[2] = {v.real(), v.imag()};
+            std::memcpy(host.data() + off + (2 * t + q) * esz, d, esz);
+        }
+}
+
+// Per radial node: the trap's kick factor and phase, and the norm's weight.
+void append_radial_nodes(gp_axial a, std::vector<char> &host) {
+    a->rad_kick = align_up(host.size(), 256);
+    a->rad_phase = align_up(a->rad_kick + a->nx * sizeof(double), 256);
+    a->line_w = align_up(a->rad_phase + a->nx * sizeof(double), 256);
+    host.resize(align_up(a->line_w + a->nx * sizeof(double), 256), 0);
+    for (int i = 0; i < a->nx; ++i) {
+        const double r = (i - 0.5) * a->drho, dv = a->dt * 0.5 * a->gamma * a->gamma * r * r;
+        const double e = std::expm1(-dv), w = i >= 1 && i <= a->nx - 2 ? 6.283185307179586 * r * a->drho * a->dz : 0.0;
+        std::memcpy(host.data() + a->rad_kick + i * sizeof(double), &e, sizeof(e));
+        std::memcpy(host.data() + a->rad_phase + i * sizeof(double), &dv, sizeof(dv));
+        std::memcpy(host.data() + a->line_w + i * sizeof(double), &w, sizeof(w));
+    }
+}
+
+// Lines per block that give every SM a block, as far as they fit (at most
+// kPcrSmem of shared memory, and at most a warp's worth of recurrences).
 template <typename R, bool CPLX> cudaError_t radial_launch(const AxArgs &args, cudaStream_t s) {
+    const size_t line = 2 * (size_t)(args.nx - 2) * sizeof(typename AxElem<R, CPLX>::V);
+    const int tl = (int)std::min<size_t>(std::min<size_t>(32, (args.nz + 151) / 152), kPcrSmem / line);
+    if (tl > 0) {
+        static bool attr = false;  // opt in once to more than 48 KB of dynamic shared memory
+        if (!attr) {
+            cudaError_t e = cudaFuncSetAttribute(axial_radial_smem_kernel<R, CPLX>,
+                                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPcrSmem);
+            if (e != cudaSuccess) return e;
+            attr = true;
+        }
+        axial_radial_smem_kernel<R, CPLX><<<(args.nz + tl - 1) / tl, kRadialThreads, tl * line, s>>>(args, tl);
+        return cudaGetLastError();
+    }
     axial_radial_kernel<R, CPLX><<<(args.nz + 127) / 128, 128, 0, s>>>(args);
     return cudaGetLastError();
 }
@@ -366,13 +528,17 @@ cudaError_t launch_radial(gp_axial a, const AxArgs &args) {
 }
 
 template <typename R, bool CPLX> cudaError_t sums_launch(const AxSums &s, cudaStream_t st) {
-    axial_sums_kernel<R, CPLX><<<kRedBlocks, kRedThreads, 0, st>>>(s);
+    const long long sites = (long long)s.nx * s.nz;
+    const unsigned blocks = (unsigned)std::min<long long>(kRedBlocks, (sites + kRedThreads - 1) / kRedThreads);
+    if (s.out) axial_sums_kernel<R, CPLX, 6><<<blocks, kRedThreads, 0, st>>>(s);
+    else axial_sums_kernel<R, CPLX, 1><<<blocks, kRedThreads, 0, st>>>(s);
     return cudaGetLastError();
 }
 
-// Cylindrical sums of the current psi (with the pending scale) -> out; with
-// scale_out, also the renormalisation factor.
+// Cylindrical sums of the current psi (with the pending scale) -> out (null:
+// the norm alone); with scale_out, also the renormalisation factor.
 gp_status queue_sums(gp_axial a, double *out, double *scale_out) {
+    const double pi = 3.141592653589793;
     AxSums s;
     s.psi = a->buf[a->cur];
     s.nx = a->nx;
@@ -380,16 +546,21 @@ gp_status queue_sums(gp_axial a, double *out, double *scale_out) {
     s.drho = a->drho;
     s.dz = a->dz;
     s.z0 = z0_of(a);
-    s.gamma2 = a->gamma * a->gamma;
-    s.lambda2 = a->lambda * a->lambda;
+    s.hg2 = 0.5 * a->gamma * a->gamma;
+    s.hl2 = 0.5 * a->lambda * a->lambda;
+    s.w0 = 2.0 * pi * a->drho * a->dz;
+    s.kr = pi * a->dz / a->drho;
+    s.kz = pi * a->drho / a->dz;
+    s.g = a->g;
     s.scale = a->d_scal + (a->scale_pending ? AS_SCALE : AS_ONE);
     s.partials = a->d_part;
+    s.counter = a->d_counter + 1;
+    s.out = out;
+    s.scale_out = scale_out;
     cudaError_t e;
     if (f32_of(a)) e = a->field == GP_COMPLEX ? sums_launch<float, true>(s, a->stream) : sums_launch<float, false>(s, a->stream);
     else e = a->field == GP_COMPLEX ? sums_launch<double, true>(s, a->stream) : sums_launch<double, false>(s, a->stream);
     AX_CK(a, e);
-    axial_finish_kernel<<<1, 32, 0, a->stream>>>(a->d_part, kRedBlocks, a->g, out, scale_out);
-    AX_CK(a, cudaGetLastError());
     return GP_OK;
 }
 
@@ -397,9 +568,17 @@ gp_status queue_sums(gp_axial a, double *out, double *scale_out) {
 // (as a pending scale).
 gp_status renormalise(gp_axial a) {
     a->scale_pending = false;  // sums of the stored values
-    gp_status st = queue_sums(a, a->d_obs + 8, a->d_scal + AS_SCALE);
+    gp_status st = queue_sums(a, nullptr, a->d_scal + AS_SCALE);
     if (st == GP_OK) a->scale_pending = true;
     return st;
+}
+
+// FP64: both sweeps by cyclic reduction where their tables exist and a line
+// fits a block's shared memory; 0 where they do not (the per-line form runs).
+int pcr_lines(gp_axial a, Form form, Kind kind, long long lines, int n, int levels) {
+    int tl = 0;
+    choose_pcr(lines, n, form, kind, levels, (int)a->elem, &tl);
+    return tl;
 }
 
 gp_status run_step(gp_axial a, bool realtime) {
@@ -422,15 +601,47 @@ gp_status run_step(gp_axial a, bool realtime) {
     r.ip = a->d_tab + a->rad_off[mode][3];
     r.scale = a->d_scal + (a->scale_pending ? AS_SCALE : AS_ONE);
     r.realtime = realtime ? 1 : 0;
-    AX_CK(a, launch_radial(a, r));
-    a->cur ^= 1;
-    a->scale_pending = false;
-    // z line solves through the Cartesian z-sweep kernels (their own norm
-    // output goes to scratch: the cylindrical one follows)
     const Geometry G = geom_of(a);
     SweepLaunch L;
     L.prec = f32_of(a) ? P_F32 : P_F64;
     L.form = realtime ? F_REALTIME : (a->field == GP_REAL ? F_IMAG_REAL : F_IMAG_CPLX);
+    const int tlr = pcr_lines(a, L.form, K_X, a->nz, a->nx - 2, a->rad_levels[mode]);
+    if (tlr > 0) {
+        SweepArgs x = sweep_args(G, 0, realtime, r.in, r.out, a->d_tab, a->T, 0, 1, r.scale, nullptr, nullptr, nullptr, nullptr);
+        if (realtime) x.phase_ex = a->d_tab + a->rad_phase;
+        else x.kick_ex = a->d_tab + a->rad_kick;
+        PcrArgs p;
+        p.levels = a->rad_levels[mode];
+        p.tl = tlr;
+        p.lv = a->d_tab + a->rad_pcr[mode][0];
+        p.im1 = a->d_tab + a->rad_pcr[mode][1];
+        p.rhs = a->d_tab + a->rad_pcr[mode][2];
+        AX_CK(a, launch_sweep_pcr(L.form, K_X, x, p, a->stream));
+    } else {
+        AX_CK(a, launch_radial(a, r));
+    }
+    a->cur ^= 1;
+    a->scale_pending = false;
+    const AxisTables &zt = a->T.ax[mode][2];
+    const int tlz = pcr_lines(a, L.form, K_Z, a->nx, a->nz - 2, zt.pcr_levels);
+    if (tlz > 0 && ((size_t)a->nx + tlz - 1) / tlz <= a->part_cap) {
+        // the z sweep carries the cylindrical norm (each row weighted by its radius)
+        SweepArgs z = sweep_args(G, 2, realtime, a->buf[a->cur], a->buf[a->cur ^ 1], a->d_tab, a->T, 0, 1,
+                                 a->d_scal + AS_ONE, a->d_part, a->d_counter, a->d_scal + AS_ZNORM, a->d_scal + AS_SCALE);
+        z.dV = 1.0;
+        PcrArgs p;
+        p.levels = zt.pcr_levels;
+        p.tl = tlz;
+        p.lv = a->d_tab + zt.off_pcr;
+        p.im1 = a->d_tab + zt.off_pcr_inv;
+        p.line_w = reinterpret_cast<const double *>(a->d_tab + a->line_w);
+        AX_CK(a, launch_sweep_pcr(L.form, K_Z, z, p, a->stream));
+        a->cur ^= 1;
+        a->scale_pending = !realtime;
+        return GP_OK;
+    }
+    // z line solves through the Cartesian z-sweep kernels (their own norm
+    // output goes to scratch: the cylindrical one follows)
     L.kind = K_Z;
     L.window = default_window(a->T.ax[mode][2], f32_of(a));
     L.threads = 64;
@@ -503,8 +714,12 @@ gp_status gp_axial_create(gp_axial *out, int nx, int nz, double drho, double dz,
     a->sites = (size_t)nx * nz;
     a->bytes = a->sites * a->elem;
     std::vector<char> host;
-    append_tables(geom_of(a), prec == GP_F32, modes_of(a), host, a->T);
+    append_tables(geom_of(a), prec == GP_F32, modes_of(a), host, a->T, kPcrAll);
     for (int mode = 0; mode < modes_of(a); ++mode) append_radial(a, mode, host);
+    if (prec == GP_F64) {
+        for (int mode = 0; mode < modes_of(a); ++mode) append_radial_pcr(a, mode, host);
+        append_radial_nodes(a, host);
+    }
     a->part_cap = std::max((size_t)kRedBlocks * 6, ((size_t)nx + 31) / 32 * (size_t)(nz > 2 ? nz - 2 : 1) + 64);
     if (dev_malloc(&a->buf[0], a->bytes) != cudaSuccess || dev_malloc(&a->buf[1], a->bytes) != cudaSuccess ||
         dev_malloc(&a->d_tab, host.size()) != cudaSuccess ||

@@ -40,7 +40,103 @@ void put_real(char *dst, double v, bool f32) {
 
 }  // namespace
 
-void append_tables(const Geometry &G, bool f32, int modes, std::vector<char> &host, Tables &T) {
+namespace {
+
+// The reduction's tables of the matrix (-a, 1 + e, -c), e the diagonal's
+// excess over one (kept apart from the one, so that 1 / D - 1 keeps its
+// relative accuracy).
+template <class Z>
+int append_pcr_t(std::vector<char> &host, std::vector<Z> a, std::vector<Z> e, std::vector<Z> c, size_t *off_lv,
+                 size_t *off_inv) {
+    const int n = (int)e.size();
+    std::vector<Z> a2(n), e2(n), c2(n), inv(n), lv;
+    a[0] = c[n - 1] = 0.0;
+    int levels = 0;
+    for (;; ++levels) {
+        double left = 0.0;
+        for (int t = 0; t < n; ++t) {
+            inv[t] = 1.0 / (1.0 + e[t]);
+            left = std::max(left, (std::abs(a[t]) + std::abs(c[t])) * std::abs(inv[t]));
+        }
+        if (levels > 0 && left <= kPcrLeft) break;
+        if (levels == kPcrMaxLevels) return 0;
+        const int d = 1 << levels;
+        for (int t = 0; t < n; ++t) {
+            const bool lo = t >= d, hi = t + d < n;
+            const Z A = lo ? a[t] * inv[t - d] : Z(0.0), C = hi ? c[t] * inv[t + d] : Z(0.0);
+            lv.push_back(A);
+            lv.push_back(C);
+            e2[t] = e[t] - (lo ? A * c[t - d] : Z(0.0)) - (hi ? C * a[t + d] : Z(0.0));
+            a2[t] = lo ? A * a[t - d] : Z(0.0);
+            c2[t] = hi ? C * c[t + d] : Z(0.0);
+        }
+        a.swap(a2);
+        e.swap(e2);
+        c.swap(c2);
+    }
+    for (int t = 0; t < n; ++t) inv[t] = -e[t] * inv[t];  // 1 / (1 + e) - 1
+    *off_lv = align_up(host.size(), 256);
+    *off_inv = align_up(*off_lv + lv.size() * sizeof(Z), 256);
+    host.resize(align_up(*off_inv + n * sizeof(Z), 256), 0);
+    std::memcpy(host.data() + *off_lv, lv.data(), lv.size() * sizeof(Z));
+    std::memcpy(host.data() + *off_inv, inv.data(), n * sizeof(Z));
+    return levels;
+}
+
+}  // namespace
+
+int append_pcr(std::vector<char> &host, const std::vector<std::complex<double>> &a,
+               const std::vector<std::complex<double>> &excess, const std::vector<std::complex<double>> &c, bool cplx,
+               size_t *off_lv, size_t *off_inv) {
+    if (cplx) return append_pcr_t<std::complex<double>>(host, a, excess, c, off_lv, off_inv);
+    auto re = [](const std::vector<std::complex<double>> &z) {
+        std::vector<double> r(z.size());
+        for (size_t t = 0; t < z.size(); ++t) r[t] = z[t].real();
+        return r;
+    };
+    return append_pcr_t<double>(host, re(a), re(excess), re(c), off_lv, off_inv);
+}
+
+// Levels that a line of constant coefficients needs: away from its ends the
+// coupling b (over the diagonal) becomes b^2 / (1 - 2 b^2) at each level.
+static int pcr_levels(std::complex<double> c) {
+    std::complex<double> b = c / (1.0 + 2.0 * c);
+    for (int l = 0; l <= kPcrMaxLevels; ++l) {
+        if (l > 0 && 2.0 * std::abs(b) <= kPcrLeft) return l;
+        b = b * b / (1.0 - 2.0 * b * b);
+    }
+    return 0;
+}
+
+// Both forms are bound by the FP64 pipe: 64 clocks per warp instruction and
+// SM sub-partition (152 SMs of four).  Thomas: a warp holds 32 lines for all
+// of its n nodes, so the busiest sub-partition has ceil(warps / 608) of them;
+// cyclic reduction spreads the nodes of a block's lines over the SM's four.
+// Operations per node and component as the kernels' forms have them (kick:
+// 12, 14, 16; norm 1 or 2).  64x48x40 real: x 62 x 18 against 8 x 24.
+bool choose_pcr(long long lines, int n, Form form, Kind kind, int levels, int elem_bytes, int *tl) {
+    if (levels < 1 || n < 1 || lines < 1 || lines > 0x7fffffffLL) return false;
+    constexpr long long kSms = 152;
+    const int extra = kind == K_X ? (form == F_IMAG_REAL ? 12 : form == F_IMAG_CPLX ? 14 : 16)
+                                  : kind == K_Z ? (form == F_IMAG_REAL ? 1 : 2) : 0;
+    const int thomas_ops = (form == F_IMAG_REAL ? 6 : form == F_IMAG_CPLX ? 12 : 16) + extra;
+    const int pcr_ops = (form == F_IMAG_REAL ? 4 + 2 * levels : form == F_IMAG_CPLX ? 8 + 4 * levels : 10 + 8 * levels) + extra;
+    auto up = [](long long a, long long b) { return (a + b - 1) / b; };
+    const long long thomas = up(up(lines, 32), 4 * kSms) * n * thomas_ops;
+    long long best = -1;
+    for (int per_sm = 1; per_sm <= 16; ++per_sm) {
+        const long long t = up(lines, kSms * per_sm);
+        if (t * n > kPcrItems || pcr_smem(elem_bytes, form == F_REALTIME ? 16 : 8, levels, (int)t, n + 2) > kPcrSmem) continue;
+        const long long cost = up(up(lines, t), kSms) * up(t * n, 128) * pcr_ops;
+        if (best < 0 || cost < best) {
+            best = cost;
+            *tl = (int)t;
+        }
+    }
+    return best >= 0 && best < thomas;
+}
+
+void append_tables(const Geometry &G, bool f32, int modes, std::vector<char> &host, Tables &T, PcrTables pcr) {
     const size_t rsz = f32 ? sizeof(float) : sizeof(double);
     const double eps = f32 ? std::ldexp(1.0, -24) : std::ldexp(1.0, -53);
     size_t off = align_up(host.size(), 256);
@@ -121,6 +217,21 @@ void append_tables(const Geometry &G, bool f32, int modes, std::vector<char> &ho
                 --at.t_const;
         }
     }
+    for (int mode = 0; pcr != kNoPcr && !f32 && mode < modes; ++mode)
+        for (int ax = 0; ax < 3; ++ax) {
+            if (G.n[ax] < 3) continue;
+            const int n = G.n[ax] - 2;
+            const double kap = G.dt / (4.0 * G.d[ax] * G.d[ax]);
+            const std::complex<double> c = mode == 1 ? std::complex<double>(0.0, kap) : std::complex<double>(kap, 0.0);
+            const Form form = mode == 1 ? F_REALTIME : modes == 2 ? F_IMAG_CPLX : F_IMAG_REAL;
+            int tl = 0;
+            if (!choose_pcr(axis_lines(G, ax), n, form, static_cast<Kind>(ax), pcr_levels(c), modes == 2 ? 16 : 8, &tl) &&
+                (pcr != kPcrAll || tl == 0))
+                continue;
+            const std::vector<std::complex<double>> off(n, c), excess(n, 2.0 * c);
+            AxisTables &at = T.ax[mode][ax];
+            at.pcr_levels = append_pcr(host, off, excess, off, mode == 1, &at.off_pcr, &at.off_pcr_inv);
+        }
 }
 
 int default_window(const AxisTables &t, bool f32) {

@@ -6,6 +6,7 @@
 
 #include "gp_internal.h"
 
+#include <complex>
 #include <string>
 #include <vector>
 
@@ -24,6 +25,8 @@ struct AxisTables {
     size_t off_cp = 0, off_ip = 0;
     int min_window = 0;   // 4, 8 or 16; 0 when none is admissible
     int t_const = 0;      // first index from which both stored tables are constant
+    int pcr_levels = 0;   // levels of the truncated cyclic reduction (0: no tables)
+    size_t off_pcr = 0, off_pcr_inv = 0;
     double cp_max = 0.0;
 };
 
@@ -36,7 +39,22 @@ struct Tables {
 
 // Append the tables of G (modes = 1: imaginary time only, 2: both) to `host`
 // (each table 256-byte aligned); offsets are relative to the start of host.
-void append_tables(const Geometry &G, bool f32, int modes, std::vector<char> &host, Tables &T);
+// With kPcrChosen also the FP64 cyclic-reduction tables of the axes that take
+// that form (choose_pcr), with kPcrAll those of every axis it can serve.
+enum PcrTables { kNoPcr, kPcrChosen, kPcrAll };
+void append_tables(const Geometry &G, bool f32, int modes, std::vector<char> &host, Tables &T, PcrTables pcr = kNoPcr);
+
+// Append FP64 cyclic-reduction tables of a line matrix (-a[t], 1 + excess[t],
+// -c[t]) to `host`: as complex values where cplx, else their real parts.
+// Returns the levels (0, and nothing appended, if kPcrMaxLevels do not reduce
+// the coupling below kPcrLeft).
+int append_pcr(std::vector<char> &host, const std::vector<std::complex<double>> &a,
+               const std::vector<std::complex<double>> &excess, const std::vector<std::complex<double>> &c, bool cplx,
+               size_t *off_lv, size_t *off_inv);
+
+// Whether an FP64 sweep of `lines` lines of n interior nodes is faster by
+// cyclic reduction than by the exact two-pass solve, and its lines per block.
+bool choose_pcr(long long lines, int n, Form form, Kind kind, int levels, int elem_bytes, int *tl);
 
 // Default window of an axis: the smallest admissible one in FP32 (bandwidth
 // bound), the exact two-pass solve (0) in FP64 (ALU bound).

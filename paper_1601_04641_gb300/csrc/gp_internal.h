@@ -86,6 +86,25 @@ struct BatchTmaMaps {
     CUtensorMap in[kTmaBatch], out[kTmaBatch];
 };
 
+// Tables and shape of a line solve by truncated cyclic reduction (gp_pcr.cuh).
+struct PcrArgs {
+    int levels;                    // reduction levels (distances 1, 2, 4, ...)
+    int tl;                        // lines per block
+    const void *lv;                // [levels][n][2]: A_l[t], C_l[t]
+    const void *im1;               // [n]: 1 / D[t] - 1 after the last level
+    const void *rhs = nullptr;     // [n][2]: A[t], C[t] of the right-hand side (radial lines), null: constant kappa
+    const double *line_w = nullptr;  // z sweep: weight of each line's |phi|^2 in the norm, null: one
+};
+constexpr int kPcrMaxLevels = 10;
+constexpr double kPcrLeft = 0x1p-55;  // coupling left after the last level: a quarter of the unit roundoff
+constexpr size_t kPcrSmem = 100 * 1024;  // most shared memory of a block: two blocks per SM
+constexpr long long kPcrItems = 8 * 1024;  // most (node, line) pairs of a block: 8 per thread
+// Two buffers of the lines' values, the tables (room for the radial form's
+// right-hand side) and a factor per line.
+inline size_t pcr_smem(int elem_bytes, int coef_bytes, int levels, int tl, int N) {
+    return (size_t)tl * (2 * (size_t)(N - 2) * elem_bytes + 8) + (size_t)(N - 2) * (2 * levels + 3) * coef_bytes;
+}
+
 struct SweepLaunch {
     Prec prec;
     Form form;
@@ -99,6 +118,8 @@ struct SweepLaunch {
 };
 
 cudaError_t launch_sweep(const SweepLaunch &L, const SweepArgs &a, cudaStream_t s);
+// FP64 line solves of one axis by truncated cyclic reduction.
+cudaError_t launch_sweep_pcr(Form form, Kind kind, const SweepArgs &a, const PcrArgs &p, cudaStream_t s);
 // Highest window the templates provide.
 constexpr int kMaxWindow = 16;
 

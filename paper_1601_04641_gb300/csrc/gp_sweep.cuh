@@ -130,6 +130,7 @@ template <typename R> __device__ __noinline__ cx<R> sincos_full(R x) {
     return r;
 }
 template <typename R> __device__ __noinline__ R expm1m_full(R y) { return g_expm1(-y); }
+__device__ __noinline__ inline double exp_full(double x) { return exp(x); }
 template <typename R> __device__ __forceinline__ void kick_sincos(R x, R *sn, R *cs) {
     if (fabs(x) <= Series<R>::kTrig) {
         Series<R>::sincos(x, sn, cs);
@@ -162,6 +163,14 @@ template <typename R> __device__ __forceinline__ R kick_apply(R q, R ex, R eyz, 
     } else {
         return fma(q, kick_dev(ex, eyz, m), q);
     }
+}
+// The same with m = exp(-y) - 1 of any size; FP64 beyond the series
+// multiplies by exp(-y) itself, which does not vanish where m rounds to -1.
+template <typename R> __device__ __forceinline__ R kick_apply_full(R q, R ex, R eyz, R y) {
+    if constexpr (sizeof(R) == 8) {
+        if (fabs(y) > Series<R>::kExp) return fma(fma(q, ex, q), eyz, fma(q, ex, q)) * exp_full(-y);
+    }
+    return kick_apply(q, ex, eyz, kick_expm1m(y));
 }
 
 // Per-site kick state of one x line.  Imaginary time: exp(-dt V) is the
@@ -239,7 +248,7 @@ template <typename R> struct FImagReal : LineForm<R> {
     __device__ __forceinline__ static R abs2(V v) { return v * v; }
     __device__ __forceinline__ static V kick(V p, const KickState<R> &k, int node) {
         const V q = p * k.s;
-        return kick_apply(q, __ldg(k.ex + node), k.eyz, kick_expm1m(k.dtg * (q * q)));
+        return kick_apply_full(q, __ldg(k.ex + node), k.eyz, k.dtg * (q * q));
     }
     // kick of NB consecutive nodes from node0: table loads issued together,
     // one series-range test per group, values equal kick's
@@ -294,8 +303,13 @@ template <typename R> struct FImagCplx : LineForm<cx<R>> {
     __device__ __forceinline__ static R abs2(V v) { return fma(v.re, v.re, v.im * v.im); }
     __device__ __forceinline__ static V kick(V p, const KickState<R> &k, int node) {
         const V q{p.re * k.s, p.im * k.s};
-        const R f = kick_dev(__ldg(k.ex + node), k.eyz, kick_expm1m(k.dtg * abs2(q)));
-        return V{fma(q.re, f, q.re), fma(q.im, f, q.im)};
+        const R y = k.dtg * abs2(q), ex = __ldg(k.ex + node);
+        if constexpr (sizeof(R) == 8) {
+            return V{kick_apply_full(q.re, ex, k.eyz, y), kick_apply_full(q.im, ex, k.eyz, y)};
+        } else {
+            const R f = kick_dev(ex, k.eyz, kick_expm1m(y));
+            return V{fma(q.re, f, q.re), fma(q.im, f, q.im)};
+        }
     }
     static constexpr bool kChunkKick = true;
     template <int NB> __device__ __forceinline__ static void kick_chunk(V (&v)[NB], const KickState<R> &k, int node0) {
