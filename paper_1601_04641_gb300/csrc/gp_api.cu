@@ -742,8 +742,7 @@ gp_status gp_init_gaussian(gp_handle h) {
     FieldArgs a = handle_field_args(h);
     const Prec p = prec_of(h);
     const bool cplx = h->field == GP_COMPLEX;
-    GP_CK(h, launch_gaussian(p, cplx, a, h->stream));
-    GP_CK(h, launch_norm(p, cplx, a, kNormBlocks, h->stream));
+    GP_CK(h, launch_gaussian(p, cplx, a, kNormBlocks, h->stream));
     h->scale_pending = true;
     h->kick_pending = false;
     h->psi_lost = false;

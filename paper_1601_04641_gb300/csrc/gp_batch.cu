@@ -595,8 +595,7 @@ gp_status gp_batch_init_gaussian(gp_batch b) {
     const bool cplx = b->field == GP_COMPLEX;
     for (int i = 0; i < b->n; ++i) {
         FieldArgs a = inst_field_args(b, i);
-        GPB_CK(b, launch_gaussian(p, cplx, a, b->stream));
-        GPB_CK(b, launch_norm(p, cplx, a, kInitNormBlocks, b->stream));
+        GPB_CK(b, launch_gaussian(p, cplx, a, kInitNormBlocks, b->stream));
         b->inst[i].step = 0;
         b->inst[i].t = 0.0;
     }

@@ -143,7 +143,8 @@ struct FieldArgs {
     unsigned int *status;  // 2 is or-ed in by an observables kernel whose bounded wait expired (may be null)
 };
 
-cudaError_t launch_gaussian(Prec p, bool cplx, const FieldArgs &a, cudaStream_t s);
+// The Gaussian and its norm (norm_out, scale_out); `blocks` as launch_norm's.
+cudaError_t launch_gaussian(Prec p, bool cplx, const FieldArgs &a, int blocks, cudaStream_t s);
 cudaError_t launch_norm(Prec p, bool cplx, const FieldArgs &a, int blocks, cudaStream_t s);
 cudaError_t launch_observables(Prec p, bool cplx, const FieldArgs &a, cudaStream_t s);
 // Look up, once per device, the launch shapes the field kernels take from

@@ -202,6 +202,53 @@ __global__ void __launch_bounds__(kReduceThreads) norm_kernel(FieldArgs a) {
         blockIdx.x, gridDim.x);
 }
 
+// The product Gaussian and its norm in one pass.  Each block evaluates the
+// three axes' factors once, (w_a/pi)^(1/4) exp(-w_a a^2/2) with zeros on the
+// boundary nodes, into shared memory; a warp then writes rows of z, one
+// product and one conversion of the FP64 pipe per site (the exponential and
+// the fourth roots per site took 200 us on a 128x96x80 grid and 13 ms of
+// setting up 64 condensates), and sums |psi|^2 of the stored values.
+constexpr int kGaussBlocks = 152 * 2;
+constexpr int kGaussAxes = 5000;  // most nodes of the three axes together: 40 KB of factors
+
+template <typename R, bool CPLX>
+__global__ void __launch_bounds__(kReduceThreads) gaussian_norm_kernel(FieldArgs a) {
+    using E = Elem<R, CPLX>;
+    extern __shared__ double factors[];
+    const int nx = a.n[0], ny = a.n[1], nz = a.n[2], lane = threadIdx.x & 31;
+    const double pi = 3.14159265358979323846;
+    for (int q = threadIdx.x; q < nx + ny + nz; q += kReduceThreads) {
+        const int ax = q < nx ? 0 : q < nx + ny ? 1 : 2, idx = q - (ax > 0 ? nx : 0) - (ax > 1 ? ny : 0);
+        const int n = a.n[ax];
+        const double x = a.origin[ax] + idx * a.d[ax];
+        // an absent axis (one node) contributes no factor and has no boundary nodes
+        factors[q] = n == 1 ? 1.0 : idx == 0 || idx == n - 1 ? 0.0 : pow(a.w[ax] / pi, 0.25) * exp(-0.5 * a.w[ax] * x * x);
+    }
+    __syncthreads();
+    typename E::V *psi = static_cast<typename E::V *>(a.psi);
+    const double *fz = factors + nx + ny;
+    double acc = 0.0;
+    const long long rows = (long long)nx * ny, warps = (long long)gridDim.x * (kReduceThreads / 32);
+    for (long long r = ((long long)blockIdx.x * kReduceThreads + threadIdx.x) >> 5; r < rows; r += warps) {
+        const int i = (int)(r / ny), j = (int)(r - (long long)i * ny);
+        const double fxy = factors[i] * factors[nx + j];
+        for (int k = lane; k < nz; k += 32) {
+            const typename E::V v = E::from_real(fxy * fz[k]);
+            psi[r * nz + k] = v;
+            acc += E::abs2(v);
+        }
+    }
+    double v[1] = {acc};
+    reduce_finalize<1>(
+        v, a,
+        [&](const double *tot) {
+            const double nrm = a.dV * tot[0];
+            *a.norm_out = nrm;
+            *a.scale_out = 1.0 / sqrt(nrm);
+        },
+        blockIdx.x, gridDim.x);
+}
+
 // Observables: one thread per (j, k) and segment of i (kObsSeg nodes) walks
 // along i.  The 9 sums (|psi|^2, V|psi|^2, |psi|^4, x^2|psi|^2, y^2|psi|^2,
 // z^2|psi|^2 and the squared forward differences to the +x, +y and +z
@@ -853,7 +900,17 @@ unsigned fill_blocks(long long sites) {
 template <typename R, bool CPLX>
 cudaError_t dispatch(int what, const FieldArgs &a, int blocks, void *dst, cudaStream_t s) {
     switch (what) {
-    case 0: gaussian_kernel<R, CPLX><<<fill_blocks(a.sites), 256, 0, s>>>(a); break;
+    case 0: {
+        const long long axes = (long long)a.n[0] + a.n[1] + a.n[2], rows = (long long)a.n[0] * a.n[1];
+        if (axes <= kGaussAxes) {
+            const unsigned g = (unsigned)std::min<long long>(kGaussBlocks, (rows + 7) / 8);
+            gaussian_norm_kernel<R, CPLX><<<g, kReduceThreads, axes * sizeof(double), s>>>(a);
+        } else {
+            gaussian_kernel<R, CPLX><<<fill_blocks(a.sites), 256, 0, s>>>(a);
+            norm_kernel<R, CPLX><<<blocks, kReduceThreads, 0, s>>>(a);
+        }
+        break;
+    }
     case 1: norm_kernel<R, CPLX><<<blocks, kReduceThreads, 0, s>>>(a); break;
     case 2:
         if constexpr (sizeof(R) == 4 && CPLX) {
@@ -931,8 +988,8 @@ int observables_blocks(const FieldArgs &a) {
     return (int)std::max(std::max((long long)observables_body_blocks(a), obs_c64z_items(a.n)), bulk);
 }
 
-cudaError_t launch_gaussian(Prec p, bool cplx, const FieldArgs &a, cudaStream_t s) {
-    return dispatch_all(p, cplx, 0, a, 0, nullptr, s);
+cudaError_t launch_gaussian(Prec p, bool cplx, const FieldArgs &a, int blocks, cudaStream_t s) {
+    return dispatch_all(p, cplx, 0, a, blocks, nullptr, s);
 }
 cudaError_t launch_norm(Prec p, bool cplx, const FieldArgs &a, int blocks, cudaStream_t s) {
     return dispatch_all(p, cplx, 1, a, blocks, nullptr, s);
