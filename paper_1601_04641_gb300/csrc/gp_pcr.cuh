@@ -185,10 +185,10 @@ __global__ void __launch_bounds__(1024) lines_pcr_kernel(SweepArgs a, PcrArgs p)
         if (tt[i] < 0) continue;
         const V r = pcr_mac(v[i], im1[tt[i]], v[i]);
         out[origin(ll[i]) + (long long)(tt[i] + 1) * a.stride] = r;
-        if (KIND == K_Z) acc = p.line_w ? fma(__ldg(p.line_w + L0 + ll[i]), F::abs2(r), acc) : acc + F::abs2(r);
+        if (KIND == K_Z && !real_time<F>()) acc = p.line_w ? fma(__ldg(p.line_w + L0 + ll[i]), F::abs2(r), acc) : acc + F::abs2(r);
     }
     // after the last level's swap y is the buffer that no thread reads any more
-    if (KIND == K_Z) pcr_norm(acc, reinterpret_cast<double *>(y), min(T, total), a);
+    if (KIND == K_Z && !real_time<F>()) pcr_norm(acc, reinterpret_cast<double *>(y), min(T, total), a);
 }
 
 template <class F, int KIND, bool RADIAL, int NS>

@@ -855,6 +855,11 @@ template <class F> struct StoreOf { using type = typename F::V; };
 template <> struct StoreOf<FImagRealH> { using type = __half; };
 template <class F> using store_t = typename StoreOf<F>::type;
 
+// Real time keeps the norm: only imaginary time's z sweeps sum it.
+template <class F> __host__ __device__ constexpr bool real_time() {
+    return std::is_same<F, FRealTime<float>>::value || std::is_same<F, FRealTime<double>>::value;
+}
+
 // The paired form of a single-line form.
 template <class F> struct PairForm { using type = FPair<F>; };
 template <> struct PairForm<FRealTime<float>> { using type = PRealTimeF; };
@@ -1201,7 +1206,7 @@ template <class F, class M, typename R, int KIND> struct Hooks {
         }
     }
     __device__ __forceinline__ void on_store(V v) const {
-        if (KIND == K_Z) acc->add(M::abs2(v));
+        if constexpr (KIND == K_Z && !real_time<F>()) acc->add(M::abs2(v));
     }
 };
 
@@ -1372,7 +1377,7 @@ template <class F, typename R, int W, int KIND, int LPT>
 __global__ void __launch_bounds__(256, 1) sweep_lines_kernel(SweepArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const double v = lines_body<F, R, W, KIND, LPT>(a, blockIdx.x, blockIdx.y, smem_raw);
-    if (KIND == K_Z) norm_finalize(v, a, blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y);
+    if (KIND == K_Z && !real_time<F>()) norm_finalize(v, a, blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y);
 }
 
 template <typename V> __host__ __device__ constexpr size_t column_ring_bytes(int threads) {
@@ -1450,12 +1455,14 @@ template <class F, typename R, int B, int W> struct TileIO {
     }
     __device__ __forceinline__ void put(int, int q, V v) {
         otile[lane * OS + q] = v;
-        csum += F::abs2(v);
+        if constexpr (!real_time<F>()) csum += F::abs2(v);
     }
     // Write positions t0 .. t0+count-1 of the 32 lines back to global memory.
     __device__ __forceinline__ void flush(int t0, int count) {
-        if (lane < nvalid) acc->add(csum);
-        csum = R(0);
+        if constexpr (!real_time<F>()) {
+            if (lane < nvalid) acc->add(csum);
+            csum = R(0);
+        }
         __syncwarp();
         if (count == B) {
             V *dst = out0 + (long long)qb * N + t0 + 1 + e;
@@ -1519,7 +1526,7 @@ template <class F, typename R, int W>
 __global__ void __launch_bounds__(kTileWarps * 32, 1) sweep_contig_kernel(SweepArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const double v = contig_body<F, R, W>(a, blockIdx.x, blockIdx.y, smem_raw);
-    norm_finalize(v, a, blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y);
+    if (!real_time<F>()) norm_finalize(v, a, blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y);
 }
 
 // ------------------------------------------------------------------ batched launches

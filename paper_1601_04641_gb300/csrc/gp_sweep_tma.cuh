@@ -251,14 +251,14 @@ __device__ __forceinline__ double tma_body(const SweepArgs &a, const CUtensorMap
 #pragma unroll
         for (int q = B - 1; q >= 0; --q) {  // result q goes to tile slot q + 1
             phi = M::back(D[q], S ? cps : ldc(cp + t0 + q), phi);
-            csum += M::abs2(phi);
+            if constexpr (!real_time<F>()) csum += M::abs2(phi);
             if (q == B - 1) next = phi;
             else if ((q & 1) == 0) hi = phi;
             else wr2(j, q + 1, phi, hi);
         }
         wr2(j, 0, carry, hi);
         carry = next;
-        acc.add(csum);
+        if constexpr (!real_time<F>()) acc.add(csum);
         store_tile(j);
 #pragma unroll
         for (int q = 0; q < W; ++q) D[q] = D[B + q];
@@ -295,10 +295,10 @@ __device__ __forceinline__ double tma_body(const SweepArgs &a, const CUtensorMap
             if (q < rem) {
                 phi = M::back(D[q], ldc(cp + t0 + q), (q == rem - 1) ? M::zero() : phi);
                 D[q] = phi;
-                csum += M::abs2(phi);
+                if constexpr (!real_time<F>()) csum += M::abs2(phi);
             }
         }
-        acc.add(csum);
+        if constexpr (!real_time<F>()) acc.add(csum);
         // tiles j, j+1, ... up to the one holding node N-1 = t0 + rem + 1
         constexpr int NT = (B + W) / B + 1;
 #pragma unroll
@@ -364,7 +364,7 @@ __global__ void __launch_bounds__(kTmaWarps * 32, 1) sweep_tma_kernel(SweepArgs 
     if (L0 < a.n_lines)
         v = tma_body<F, R, W>(a, &maps.in, &maps.out, base + warp * S * kTmaBoxBytes,
                               smem_u32(base + kTmaWarps * S * kTmaBoxBytes) + 8 * S * warp, (int)L0);
-    norm_finalize(v, a, blockIdx.x, gridDim.x);
+    if (!real_time<F>()) norm_finalize(v, a, blockIdx.x, gridDim.x);
 }
 
 // ------------------------------------------------------------------ strided axes through TMA
