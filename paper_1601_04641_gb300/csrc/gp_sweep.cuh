@@ -953,7 +953,8 @@ __device__ __forceinline__ void cp_async_wait(int pending) {
 // Outputs per chunk of the windowed solve: 16, or 8 for 16-byte elements
 // (complex FP64) to bound the register ring.
 template <typename V> __host__ __device__ constexpr int chunk_len() { return sizeof(V) >= 16 ? 8 : 16; }
-// Chunks in a line's input ring: two readable, two in flight.
+// Chunks in the input ring of the contiguous axis and the box forms: two
+// readable, two in flight.
 constexpr int kRingChunks = 4;
 
 // Windowed Thomas solve of the interior nodes [tb, te) of a line of n
@@ -1010,10 +1011,15 @@ __device__ __forceinline__ void solve_segment(int n, int tb, int te, int tconst,
     // the segment behaves as a line ending at e: W look-ahead values beyond
     // te start the windowed backward sweep of its last chunk
     const int e = min(te + W, n);
-    io.start(tw - 1, e + 2);
-    io.need(tw + 2);
-    V pm = io.val(tw - 1);
+    io.start(tw - 1, e + 2, tb);
+    V pm = F::zero();
+    if (tw > 0) {
+        io.need(tw);
+        pm = io.val(tw - 1);
+    }
+    io.need(tw + 1);
     V p0 = io.val(tw);
+    io.need(tw + 2);
     V p1 = io.val(tw + 1);
     V dprev = F::zero();
     for (int t = tw; t < tb; ++t) {
@@ -1254,59 +1260,71 @@ template <class F, class M, typename R, int KIND> struct DirectIO {
 // One thread owns one segment of one line (element stride st); consecutive
 // threads own lines adjacent in memory, so each cp.async instruction of a
 // warp reads one contiguous row.  Each thread streams its line through a
-// private column of a shared ring, ring[position % R][thread], R = 4 chunks:
-// while one chunk is consumed the next two are in flight.
-template <class F, class M, typename R, int B, int KIND> struct ColumnIO {
+// private column of a shared ring of three chunks.  The chunks start where an
+// output chunk's inputs do (position t0 + W + 2), so that an output chunk
+// reads exactly one of them, at fixed offsets from its slot, while the next
+// two are in flight.  TB is the block size (0: taken at run time); fixed, the
+// ring's offsets are immediates.  (A ring of four chunks from the segment's
+// first position, masked per node, spent 20 integer instructions per site on
+// the complex64 x sweep.)
+constexpr int kColumnChunks = 3;
+template <class F, class M, typename R, int B, int W, int KIND, int TB> struct ColumnIO {
     using V = typename M::V;
     using MV = typename M::MemV;
-    static constexpr int RL = kRingChunks * B;  // ring length (power of two)
     const MV *in;
     MV *out;
-    MV *ring;     // this thread's column: element p at ring[(p - s0) % RL * T]
+    MV *ring;       // this thread's column: node e of slot s at ring[(s B + e) T]
+    const MV *src;  // node of the next chunk's first position
     long long st;
-    int n, T, s0, limit, issued, ready;
+    int n, blk, s0, first, limit, issued, ready, wslot;
     Hooks<F, M, R, KIND> hk;
+    __device__ __forceinline__ int T() const { return TB > 0 ? TB : blk; }
     __device__ __forceinline__ void issue() {
         const int pb = s0 + issued * B;
-        // the chunk's B ring rows are consecutive: (pb + e - s0) mod RL =
-        // ((issued B) mod RL) + e, since RL is a multiple of B
-        MV *slot = ring + ((issued * B) & (RL - 1)) * T;
-        if (pb >= 0 && pb + B <= n) {
-            // the whole chunk inside the line (every chunk but a line's
-            // first and last): no per-element range test or select
-            const MV *g = in + (long long)(pb + 1) * st;
+        MV *slot = ring + wslot * (B * T());
+        if (pb >= max(first, 0) && pb + B <= n) {
+            // the whole chunk inside the line and the segment's reach (every
+            // chunk but the first and the last): no per-element range test
 #pragma unroll
-            for (int e = 0; e < B; ++e) cp_async<sizeof(MV)>(slot + e * T, g + e * st, true);
+            for (int e = 0; e < B; ++e) cp_async<sizeof(MV)>(slot + e * T(), src + e * st, true);
         } else {
 #pragma unroll
             for (int e = 0; e < B; ++e) {
                 const int p = pb + e;
-                const bool ok = p >= 0 && p < n;
-                cp_async<sizeof(MV)>(slot + e * T, ok ? in + (long long)(p + 1) * st : in, ok);
+                const bool ok = p >= max(first, 0) && p < n;
+                cp_async<sizeof(MV)>(slot + e * T(), ok ? src + e * st : in, ok);
             }
         }
         cp_async_commit();
         ++issued;
+        src += B * st;
+        wslot = wslot == kColumnChunks - 1 ? 0 : wslot + 1;
     }
-    __device__ __forceinline__ void start(int first, int lim) {
-        s0 = first;
+    __device__ __forceinline__ void start(int f, int lim, int tb) {
+        s0 = tb + W + 2 - (2 * W + 4 + B - 1) / B * B;
+        if (f > s0) s0 += (f - s0) / B * B;
+        first = f;
         limit = lim;
-        issued = ready = 0;
-        while (issued < kRingChunks - 1 && s0 + issued * B < limit) issue();
+        issued = ready = wslot = 0;
+        src = in + (long long)(s0 + 1) * st;
+        while (issued < kColumnChunks && s0 + issued * B < limit) issue();
     }
     __device__ __forceinline__ void need(int p_end) {
         const int c = (p_end - 1 - s0) / B;
         if (c < ready) return;
         cp_async_wait(issued - 1 - c);
         ready = c + 1;
-        while (issued <= c + kRingChunks - 2 && s0 + issued * B < limit) issue();
+        while (issued < c + kColumnChunks && s0 + issued * B < limit) issue();  // over the chunks before c
     }
     __device__ __forceinline__ V val(int p) const {
-        return hk.on_load(p, M::load(ring[((p - s0) & (RL - 1)) * T]));
+        const int q = p - s0, c = q / B;
+        return hk.on_load(p, M::load(ring[((c % kColumnChunks) * B + (q - c * B)) * T()]));
     }
     template <int NB> __device__ __forceinline__ void vals(int p, V (&v)[NB]) const {
+        static_assert(NB == B, "an output chunk reads one chunk of the ring");
+        const MV *slot = ring + ((p - s0) / B % kColumnChunks) * (B * T());
 #pragma unroll
-        for (int q = 0; q < NB; ++q) v[q] = M::load(ring[((p + q - s0) & (RL - 1)) * T]);
+        for (int q = 0; q < NB; ++q) v[q] = M::load(slot[q * T()]);
         hk.on_load_chunk(p, v);
     }
     __device__ __forceinline__ void put(int t0, int q, V v) const {
@@ -1323,7 +1341,7 @@ template <class F> struct LinesPerThread<F, 4> { using M = typename QuadForm<F>:
 // One thread per (line, segment), or per (group of LPT = 2 or 4 adjacent
 // lines, segment); blockIdx.y is the segment.  Window 0 selects the exact
 // two-pass form over whole lines with direct access.
-template <class F, typename R, int W, int KIND, int LPT>
+template <class F, typename R, int W, int KIND, int LPT, int TB>
 __device__ __forceinline__ double lines_body(const SweepArgs &a, unsigned bx, unsigned seg,
                                              unsigned char *smem_raw) {
     using M = typename LinesPerThread<F, LPT>::M;
@@ -1344,12 +1362,12 @@ __device__ __forceinline__ double lines_body(const SweepArgs &a, unsigned bx, un
         if (seg == 0) out[0] = M::store(M::zero());
         if ((int)seg == a.n_seg - 1) out[(long long)(a.N - 1) * st] = M::store(M::zero());
         if constexpr (W > 0) {
-            ColumnIO<F, M, R, B, KIND> io;
+            ColumnIO<F, M, R, B, W, KIND, TB> io;
             io.in = in;
             io.out = out;
             io.st = st;
             io.n = n;
-            io.T = blockDim.x;
+            io.blk = blockDim.x;
             io.ring = reinterpret_cast<MV *>(smem_raw) + threadIdx.x;
             io.hk.acc = &acc;
             io.hk.init(a, L);
@@ -1373,15 +1391,16 @@ __device__ __forceinline__ double lines_body(const SweepArgs &a, unsigned bx, un
 // One thread per (line, segment), or per (pair of adjacent lines, segment)
 // when LPT = 2; blockIdx.y is the segment.  Window 0 selects the exact
 // two-pass form over whole lines with direct access.
-template <class F, typename R, int W, int KIND, int LPT>
-__global__ void __launch_bounds__(256, 1) sweep_lines_kernel(SweepArgs a) {
+// TB: threads per block, 0 for any.
+template <class F, typename R, int W, int KIND, int LPT, int TB>
+__global__ void __launch_bounds__(TB > 0 ? TB : 256, 1) sweep_lines_kernel(SweepArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const double v = lines_body<F, R, W, KIND, LPT>(a, blockIdx.x, blockIdx.y, smem_raw);
+    const double v = lines_body<F, R, W, KIND, LPT, TB>(a, blockIdx.x, blockIdx.y, smem_raw);
     if (KIND == K_Z && !real_time<F>()) norm_finalize(v, a, blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y);
 }
 
 template <typename V> __host__ __device__ constexpr size_t column_ring_bytes(int threads) {
-    return (size_t)kRingChunks * chunk_len<V>() * threads * sizeof(V);
+    return (size_t)kColumnChunks * chunk_len<V>() * threads * sizeof(V);
 }
 
 // ------------------------------------------------------------------ contiguous axis
@@ -1433,7 +1452,7 @@ template <class F, typename R, int B, int W> struct TileIO {
         cp_async_commit();
         ++issued;
     }
-    __device__ __forceinline__ void start(int first, int lim) {
+    __device__ __forceinline__ void start(int first, int lim, int) {
         s0 = first;
         limit = lim;
         issued = ready = 0;
@@ -1552,14 +1571,14 @@ __device__ __forceinline__ int find_instance(const BatchDesc &d, unsigned b) {
 }
 
 template <class F, typename R, int W, int KIND, int LPT>
-__global__ void __launch_bounds__(256, 1) batch_lines_kernel(BatchDesc d) {
+__global__ void __launch_bounds__(kBatchLineThreads, 1) batch_lines_kernel(BatchDesc d) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int i = find_instance(d, blockIdx.x);
     const SweepArgs a = d.args[i];
     const unsigned local = blockIdx.x - __ldg(d.first + i);
     const unsigned gx = __ldg(d.gridx + i);
     const unsigned nblocks = __ldg(d.first + i + 1) - __ldg(d.first + i);
-    const double v = lines_body<F, R, W, KIND, LPT>(a, local % gx, local / gx, smem_raw);
+    const double v = lines_body<F, R, W, KIND, LPT, kBatchLineThreads>(a, local % gx, local / gx, smem_raw);
     if (KIND == K_Z) norm_finalize(v, a, local, nblocks);
 }
 

@@ -414,7 +414,7 @@ template <class F, class M, typename R, int B, int KIND> struct TmaColumnIO {
         }
         ++issued;
     }
-    __device__ __forceinline__ void start(int first, int lim) {
+    __device__ __forceinline__ void start(int first, int lim, int) {
         s0 = first;
         limit = lim;
         issued = ready = 0;

@@ -94,14 +94,23 @@ static cudaError_t launch_lines_wl_any(const SweepLaunch &L, const SweepArgs &a,
     const long long units = (a.n_lines + LPT - 1) / LPT;
     const dim3 grid((unsigned)((units + threads - 1) / threads), (unsigned)a.n_seg);
     const size_t smem = W > 0 ? column_ring_bytes<V>(threads) : 0;
+    // FP32 at its usual block size: the form with that size fixed
+    constexpr int TB = W > 0 && KIND != K_Z && sizeof(R) == 4 ? kBatchLineThreads : 0;
+    if constexpr (TB > 0) {
+        if (threads == TB) {
+            static_assert(column_ring_bytes<V>(TB) <= 48 * 1024, "no opt-in to more shared memory");
+            sweep_lines_kernel<F, R, W, KIND, LPT, TB><<<grid, threads, smem, s>>>(a);
+            return cudaGetLastError();
+        }
+    }
     static int attr = 0;  // largest dynamic shared memory opted in so far
     if ((int)smem > attr && smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(sweep_lines_kernel<F, R, W, KIND, LPT>,
+        cudaError_t e = cudaFuncSetAttribute(sweep_lines_kernel<F, R, W, KIND, LPT, 0>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         attr = (int)smem;
     }
-    sweep_lines_kernel<F, R, W, KIND, LPT><<<grid, threads, smem, s>>>(a);
+    sweep_lines_kernel<F, R, W, KIND, LPT, 0><<<grid, threads, smem, s>>>(a);
     return cudaGetLastError();
 }
 
