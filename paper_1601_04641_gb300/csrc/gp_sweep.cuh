@@ -1391,9 +1391,19 @@ __device__ __forceinline__ double lines_body(const SweepArgs &a, unsigned bx, un
 // One thread per (line, segment), or per (pair of adjacent lines, segment)
 // when LPT = 2; blockIdx.y is the segment.  Window 0 selects the exact
 // two-pass form over whole lines with direct access.
+// Blocks of 64 threads per SM that the compiler leaves registers for: eight
+// (128 registers, no spills) for single FP32 lines of windows 4 and 8, whose
+// rings leave room for as many (241x201x161 complex64 imaginary time 1.29 ->
+// 1.17 ms per 10 steps).  Line groups keep theirs: held to 128, complex64 real
+// time gained 1 % on 480x400x320 and lost 4 % on 200x160x120, where two blocks
+// an SM are all there are; wider windows spill.
+template <class F, int W, int LPT> __host__ __device__ constexpr int lines_min_blocks() {
+    return sizeof(typename F::Real) == 4 && (W == 4 || W == 8) && LPT == 1 ? 8 : 1;
+}
+
 // TB: threads per block, 0 for any.
 template <class F, typename R, int W, int KIND, int LPT, int TB>
-__global__ void __launch_bounds__(TB > 0 ? TB : 256, 1) sweep_lines_kernel(SweepArgs a) {
+__global__ void __launch_bounds__(TB > 0 ? TB : 256, TB > 0 ? lines_min_blocks<F, W, LPT>() : 1) sweep_lines_kernel(SweepArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const double v = lines_body<F, R, W, KIND, LPT, TB>(a, blockIdx.x, blockIdx.y, smem_raw);
     if (KIND == K_Z && !real_time<F>()) norm_finalize(v, a, blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y);
@@ -1571,7 +1581,7 @@ __device__ __forceinline__ int find_instance(const BatchDesc &d, unsigned b) {
 }
 
 template <class F, typename R, int W, int KIND, int LPT>
-__global__ void __launch_bounds__(kBatchLineThreads, 1) batch_lines_kernel(BatchDesc d) {
+__global__ void __launch_bounds__(kBatchLineThreads, lines_min_blocks<F, W, LPT>()) batch_lines_kernel(BatchDesc d) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int i = find_instance(d, blockIdx.x);
     const SweepArgs a = d.args[i];
