@@ -240,23 +240,51 @@ gp_status build_set(gp_batch b) {
     LaunchSet &S = b->act;
     for (int i = 0; i < b->n; ++i)
         if (b->inst[i].active) S.members.push_back(i);
-    // stream groups balanced by sites: largest instance first to the least
-    // loaded group
-    const int ng = std::max(1, std::min(b->streams, (int)S.members.size()));
-    std::vector<std::vector<int>> groups(ng);
+    // stream groups: instances that take the same launches (lines per thread
+    // on x and y, the z sweep's form) share groups, so that a group's step is
+    // one launch per sweep wherever there are groups enough; the groups of a
+    // kind (about its share of the sites) are balanced by sites, largest
+    // instance first to the least loaded
+    int ng = std::max(1, std::min(b->streams, (int)S.members.size()));
+    std::vector<std::vector<int>> groups;
     {
-        std::vector<int> bysize(S.members);
-        std::stable_sort(bysize.begin(), bysize.end(),
-                         [&](int a, int c) { return b->inst[a].sites > b->inst[c].sites; });
-        std::vector<size_t> load(ng, 0);
-        for (int i : bysize) {
-            const int gi = (int)(std::min_element(load.begin(), load.end()) - load.begin());
-            groups[gi].push_back(i);
-            load[gi] += b->inst[i].sites;
+        std::map<int, std::vector<int>> kinds;
+        std::map<int, size_t> weight;
+        size_t all = 0;
+        for (int i : S.members) {
+            const Inst &I = b->inst[i];
+            const int kind = I.lpt[0] + 4 * I.lpt[1] + (I.ztma ? 16 : 0);
+            kinds[kind].push_back(i);
+            weight[kind] += I.sites;
+            all += I.sites;
         }
+        // asked for concurrent groups at all, every kind gets one
+        if (b->streams > 1) ng = std::max(ng, (int)kinds.size());
+        groups.resize(ng);
+        std::vector<int> order;
+        for (auto &kv : kinds) order.push_back(kv.first);
+        std::stable_sort(order.begin(), order.end(), [&](int a, int c) { return weight[a] > weight[c]; });
+        std::vector<size_t> load(ng, 0);
+        int used = 0;
+        for (size_t q = 0; q < order.size(); ++q) {
+            const int left = (int)(order.size() - q) - 1;  // kinds still to come keep a group each, while there are any
+            const int want = (int)((double)ng * (double)weight[order[q]] / (double)all + 0.5);
+            const int take = std::max(0, std::min(std::max(1, q + 1 == order.size() ? ng - used : want), ng - used - left));
+            std::vector<int> &v = kinds[order[q]];
+            std::stable_sort(v.begin(), v.end(), [&](int a, int c) { return b->inst[a].sites > b->inst[c].sites; });
+            const int g0 = take > 0 ? used : 0, g1 = take > 0 ? used + take : std::max(1, used);
+            for (int i : v) {
+                const int gi = (int)(std::min_element(load.begin() + g0, load.begin() + g1) - load.begin());
+                groups[gi].push_back(i);
+                load[gi] += b->inst[i].sites;
+            }
+            used += take;
+        }
+        groups.erase(std::remove_if(groups.begin(), groups.end(), [](const std::vector<int> &g) { return g.empty(); }),
+                     groups.end());
     }
-    S.sets.assign(ng, SweepSet());
-    for (int gs = 0; gs < ng; ++gs) {
+    S.sets.assign(groups.size(), SweepSet());
+    for (size_t gs = 0; gs < groups.size(); ++gs) {
         SweepSet &T = S.sets[gs];
         T.zmaps.assign(2, BatchTmaMaps());
         for (int k = 0; k < 3; ++k) {

@@ -1260,17 +1260,26 @@ template <class F, class M, typename R, int KIND> struct DirectIO {
 // One thread owns one segment of one line (element stride st); consecutive
 // threads own lines adjacent in memory, so each cp.async instruction of a
 // warp reads one contiguous row.  Each thread streams its line through a
-// private column of a shared ring of three chunks.  The chunks start where an
-// output chunk's inputs do (position t0 + W + 2), so that an output chunk
-// reads exactly one of them, at fixed offsets from its slot, while the next
-// two are in flight.  TB is the block size (0: taken at run time); fixed, the
-// ring's offsets are immediates.  (A ring of four chunks from the segment's
-// first position, masked per node, spent 20 integer instructions per site on
-// the complex64 x sweep.)
-constexpr int kColumnChunks = 3;
+// private column of a shared ring of chunks.
+// Aligned: three chunks, which start where an output chunk's inputs do
+// (position t0 + W + 2), so that an output chunk reads exactly one of them, at
+// fixed offsets from its slot, while the next two are in flight.  TB is the
+// block size (0: taken at run time); fixed, the ring's offsets are immediates.
+// (A ring of four chunks from the segment's first position, masked per node,
+// spent 20 integer instructions per site on the complex64 x sweep.)
+// Where that start lies 12 nodes before the segment's first input (chunks of
+// 16, windows 8 and 16), a short line would wait for one more chunk (64 FP32
+// real condensates at window 16: 0.229 -> 0.237 ms a step): those forms keep
+// the ring of four from the first position.
+template <int B, int W> __host__ __device__ constexpr bool column_aligned() {
+    return (2 * W + 4 + B - 1) / B * B - (2 * W + 4) <= 4;
+}
+template <int B, int W> __host__ __device__ constexpr int column_chunks() { return column_aligned<B, W>() ? 3 : 4; }
 template <class F, class M, typename R, int B, int W, int KIND, int TB> struct ColumnIO {
     using V = typename M::V;
     using MV = typename M::MemV;
+    static constexpr bool ALIGNED = column_aligned<B, W>();
+    static constexpr int RC = column_chunks<B, W>();
     const MV *in;
     MV *out;
     MV *ring;       // this thread's column: node e of slot s at ring[(s B + e) T]
@@ -1298,33 +1307,41 @@ template <class F, class M, typename R, int B, int W, int KIND, int TB> struct C
         cp_async_commit();
         ++issued;
         src += B * st;
-        wslot = wslot == kColumnChunks - 1 ? 0 : wslot + 1;
+        wslot = wslot == RC - 1 ? 0 : wslot + 1;
     }
     __device__ __forceinline__ void start(int f, int lim, int tb) {
-        s0 = tb + W + 2 - (2 * W + 4 + B - 1) / B * B;
-        if (f > s0) s0 += (f - s0) / B * B;
+        s0 = f;
+        if (ALIGNED) {
+            s0 = tb + W + 2 - (2 * W + 4 + B - 1) / B * B;
+            if (f > s0) s0 += (f - s0) / B * B;
+        }
         first = f;
         limit = lim;
         issued = ready = wslot = 0;
         src = in + (long long)(s0 + 1) * st;
-        while (issued < kColumnChunks && s0 + issued * B < limit) issue();
+        while (issued < 3 && s0 + issued * B < limit) issue();
     }
     __device__ __forceinline__ void need(int p_end) {
         const int c = (p_end - 1 - s0) / B;
         if (c < ready) return;
         cp_async_wait(issued - 1 - c);
         ready = c + 1;
-        while (issued < c + kColumnChunks && s0 + issued * B < limit) issue();  // over the chunks before c
+        while (issued < c + 3 && s0 + issued * B < limit) issue();  // over chunks that nothing reads any more
     }
     __device__ __forceinline__ V val(int p) const {
         const int q = p - s0, c = q / B;
-        return hk.on_load(p, M::load(ring[((c % kColumnChunks) * B + (q - c * B)) * T()]));
+        return hk.on_load(p, M::load(ring[((c % RC) * B + (q - c * B)) * T()]));
     }
     template <int NB> __device__ __forceinline__ void vals(int p, V (&v)[NB]) const {
-        static_assert(NB == B, "an output chunk reads one chunk of the ring");
-        const MV *slot = ring + ((p - s0) / B % kColumnChunks) * (B * T());
+        if constexpr (ALIGNED) {
+            static_assert(NB == B, "an output chunk reads one chunk of the ring");
+            const MV *slot = ring + ((p - s0) / B % RC) * (B * T());
 #pragma unroll
-        for (int q = 0; q < NB; ++q) v[q] = M::load(slot[q * T()]);
+            for (int q = 0; q < NB; ++q) v[q] = M::load(slot[q * T()]);
+        } else {
+#pragma unroll
+            for (int q = 0; q < NB; ++q) v[q] = M::load(ring[((p + q - s0) & (RC * B - 1)) * T()]);
+        }
         hk.on_load_chunk(p, v);
     }
     __device__ __forceinline__ void put(int t0, int q, V v) const {
@@ -1409,8 +1426,8 @@ __global__ void __launch_bounds__(TB > 0 ? TB : 256, TB > 0 ? lines_min_blocks<F
     if (KIND == K_Z && !real_time<F>()) norm_finalize(v, a, blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y);
 }
 
-template <typename V> __host__ __device__ constexpr size_t column_ring_bytes(int threads) {
-    return (size_t)kColumnChunks * chunk_len<V>() * threads * sizeof(V);
+template <typename V, int W> __host__ __device__ constexpr size_t column_ring_bytes(int threads) {
+    return (size_t)column_chunks<chunk_len<V>(), W>() * chunk_len<V>() * threads * sizeof(V);
 }
 
 // ------------------------------------------------------------------ contiguous axis

@@ -93,12 +93,12 @@ static cudaError_t launch_lines_wl_any(const SweepLaunch &L, const SweepArgs &a,
     const unsigned threads = (unsigned)L.threads;
     const long long units = (a.n_lines + LPT - 1) / LPT;
     const dim3 grid((unsigned)((units + threads - 1) / threads), (unsigned)a.n_seg);
-    const size_t smem = W > 0 ? column_ring_bytes<V>(threads) : 0;
+    const size_t smem = W > 0 ? column_ring_bytes<V, W>(threads) : 0;
     // FP32 at its usual block size: the form with that size fixed
     constexpr int TB = W > 0 && KIND != K_Z && sizeof(R) == 4 ? kBatchLineThreads : 0;
     if constexpr (TB > 0) {
         if (threads == TB) {
-            static_assert(column_ring_bytes<V>(TB) <= 48 * 1024, "no opt-in to more shared memory");
+            static_assert(column_ring_bytes<V, W>(TB) <= 48 * 1024, "no opt-in to more shared memory");
             sweep_lines_kernel<F, R, W, KIND, LPT, TB><<<grid, threads, smem, s>>>(a);
             return cudaGetLastError();
         }
@@ -152,7 +152,7 @@ template <class F, typename R, int W, int KIND, int LPT>
 static cudaError_t launch_batch_lines_wl(const BatchLaunch &b, cudaStream_t s) {
     using V = typename LinesPerThread<F, LPT>::M::MemV;
     const unsigned threads = kBatchLineThreads;
-    const size_t smem = W > 0 ? column_ring_bytes<V>(threads) : 0;
+    const size_t smem = W > 0 ? column_ring_bytes<V, W>(threads) : 0;
     static bool attr = false;
     if (!attr && smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(batch_lines_kernel<F, R, W, KIND, LPT>,
