@@ -611,6 +611,7 @@ gp_status run_step(gp_axial a, bool realtime) {
         if (realtime) x.phase_ex = a->d_tab + a->rad_phase;
         else x.kick_ex = a->d_tab + a->rad_kick;
         PcrArgs p;
+        p.dependent = true;
         p.levels = a->rad_levels[mode];
         p.tl = tlr;
         p.lv = a->d_tab + a->rad_pcr[mode][0];
@@ -630,6 +631,7 @@ gp_status run_step(gp_axial a, bool realtime) {
                                  a->d_scal + AS_ONE, a->d_part, a->d_counter, a->d_scal + AS_ZNORM, a->d_scal + AS_SCALE);
         z.dV = 1.0;
         PcrArgs p;
+        p.dependent = true;
         p.levels = zt.pcr_levels;
         p.tl = tlz;
         p.lv = a->d_tab + zt.off_pcr;

@@ -93,6 +93,7 @@ struct PcrArgs {
     const void *lv;                // [levels][n][2]: A_l[t], C_l[t]
     const void *im1;               // [n]: 1 / D[t] - 1 after the last level
     const void *rhs = nullptr;     // [n][2]: A[t], C[t] of the right-hand side (radial lines), null: constant kappa
+    bool dependent = false;        // launched as a programmatic dependent (not into graph captures)
     const double *line_w = nullptr;  // z sweep: weight of each line's |phi|^2 in the norm, null: one
 };
 constexpr int kPcrMaxLevels = 10;

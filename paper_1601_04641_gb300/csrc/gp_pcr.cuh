@@ -23,6 +23,7 @@
 // its better balance outweighs that (choose_pcr).
 #pragma once
 
+#include "gp_async.cuh"
 #include "gp_sweep.cuh"
 
 namespace gpcn {
@@ -110,6 +111,13 @@ __global__ void __launch_bounds__(1024) lines_pcr_kernel(SweepArgs a, PcrArgs p)
         const unsigned o = L / (unsigned)a.inner;
         return (long long)o * a.outer_stride + (L - o * (unsigned)a.inner);
     };
+    // the tables, which no launch writes, while the previous sweep ends
+    pdl_trigger();
+    for (int q = threadIdx.x; q < ntab; q += T) tab[q] = ldc(static_cast<const C *>(p.lv) + q);
+    for (int q = threadIdx.x; q < n; q += T) im1[q] = ldc(static_cast<const C *>(p.im1) + q);
+    if (RADIAL)
+        for (int q = threadIdx.x; q < 2 * n; q += T) rhs[q] = ldc(static_cast<const C *>(p.rhs) + q);
+    pdl_wait();
     // item i of the thread: node t of line l of the block (the global
     // accesses of a warp run along the contiguous axis), all ones past the end
     int tt[NS], ll[NS];
@@ -136,10 +144,6 @@ __global__ void __launch_bounds__(1024) lines_pcr_kernel(SweepArgs a, PcrArgs p)
                 v[i] = in[origin(ll[i]) + (long long)(tt[i] + 1) * a.stride];
         }
     }
-    for (int q = threadIdx.x; q < ntab; q += T) tab[q] = ldc(static_cast<const C *>(p.lv) + q);
-    for (int q = threadIdx.x; q < n; q += T) im1[q] = ldc(static_cast<const C *>(p.im1) + q);
-    if (RADIAL)
-        for (int q = threadIdx.x; q < 2 * n; q += T) rhs[q] = ldc(static_cast<const C *>(p.rhs) + q);
     for (int q = threadIdx.x; q < 2 * nl; q += T)  // the line ends
         out[origin(q >> 1) + (q & 1 ? (long long)(a.N - 1) * a.stride : 0)] = F::zero();
     if (KIND == K_X) __syncthreads();  // lk
@@ -201,6 +205,7 @@ inline cudaError_t launch_pcr_ns(const SweepArgs &a, const PcrArgs &p, int threa
         if (e != cudaSuccess) return e;
         attr = true;
     }
+    if (p.dependent) return launch_dependent(lines_pcr_kernel<F, KIND, RADIAL, NS>, grid, threads, smem, s, a, p);
     lines_pcr_kernel<F, KIND, RADIAL, NS><<<grid, threads, smem, s>>>(a, p);
     return cudaGetLastError();
 }
