@@ -22,6 +22,9 @@ struct gp_nn_s {
     const float *data = nullptr;
     float *d_grad = nullptr, *d_loss = nullptr, *d_partials = nullptr, *d_lpart = nullptr;
     int part_blocks = 0;
+    int *d_si = nullptr;           // explicit samples (gp_nn_loss_grad): instances and sites, kept from call to call
+    long long *d_ss = nullptr;
+    int sample_cap = 0;
     long long adam_t = 0;
     std::string err;
 };
@@ -62,6 +65,24 @@ gp_status ensure_partials(gp_nn net, int blocks) {
         return nfail(net, GP_ERR_NOMEM, "cudaMalloc of gradient partials failed");
     }
     net->part_blocks = blocks;
+    return GP_OK;
+}
+
+// Room for `count` explicit samples (a training program evaluates batch after
+// batch of one size: the buffers are allocated once and grow with it).
+gp_status ensure_samples(gp_nn net, int count) {
+    if (count <= net->sample_cap) return GP_OK;
+    cudaFree(net->d_si);
+    cudaFree(net->d_ss);
+    net->d_si = nullptr;
+    net->d_ss = nullptr;
+    net->sample_cap = 0;
+    if (gpcn::dev_malloc(&net->d_si, count * sizeof(int)) != cudaSuccess ||
+        gpcn::dev_malloc(&net->d_ss, count * sizeof(long long)) != cudaSuccess) {
+        cudaGetLastError();
+        return nfail(net, GP_ERR_NOMEM, "cudaMalloc of the samples failed");
+    }
+    net->sample_cap = count;
     return GP_OK;
 }
 
@@ -162,6 +183,8 @@ void gp_nn_destroy(gp_nn net) {
     cudaFree(net->d_loss);
     cudaFree(net->d_partials);
     cudaFree(net->d_lpart);
+    cudaFree(net->d_si);
+    cudaFree(net->d_ss);
     cudaGetLastError();
     delete net;
 }
@@ -262,13 +285,9 @@ gp_status gp_nn_loss_grad(gp_nn net, int count, const int *instance, const long 
             return nfail(net, GP_ERR_ARG, "sample out of range");
     const int blocks = count / 128;
     if ((st = ensure_partials(net, blocks)) != GP_OK) return st;
-    int *d_i = nullptr;
-    long long *d_s = nullptr;
-    if (gpcn::dev_malloc(&d_i, count * sizeof(int)) != cudaSuccess || gpcn::dev_malloc(&d_s, count * sizeof(long long)) != cudaSuccess) {
-        cudaGetLastError();
-        cudaFree(d_i);
-        return nfail(net, GP_ERR_NOMEM, "cudaMalloc of the samples failed");
-    }
+    if ((st = ensure_samples(net, count)) != GP_OK) return st;
+    int *d_i = net->d_si;
+    long long *d_s = net->d_ss;
     NNTrain T{};
     T.inst = net->d_inst;
     T.n_inst = net->n_inst;
@@ -286,9 +305,9 @@ gp_status gp_nn_loss_grad(gp_nn net, int count, const int *instance, const long 
     if (e == cudaSuccess && grad)
         e = cudaMemcpyAsync(grad, net->d_grad, kNNParams * sizeof(float), cudaMemcpyDeviceToHost, net->stream);
     if (e == cudaSuccess && loss) e = cudaMemcpyAsync(loss, net->d_loss, sizeof(float), cudaMemcpyDeviceToHost, net->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(net->stream);
-    cudaFree(d_i);
-    cudaFree(d_s);
+    // also on an error: the copies read the caller's arrays
+    const cudaError_t es = cudaStreamSynchronize(net->stream);
+    if (e == cudaSuccess) e = es;
     if (e != cudaSuccess) return nfail(net, GP_ERR_CUDA, std::string("gradient evaluation failed: ") + cudaGetErrorString(e));
     return GP_OK;
 }

@@ -13,7 +13,7 @@
 //   d2 = (d3 W2^T)(1 - h2^2),  d1 = (d2 W1^T)(1 - h1^2),
 //   dW2 = h2^T d3, dW1 = h1^T d2, dW0 = x^T d1 (tensor cores, K = points),
 //   biases: column sums of d; dw3 = h3^T dz4; db3 = sum dz4,
-// written as per-block partial gradients, summed in block order by a second
+// written as per-block partial gradients, summed in a fixed grouping by a second
 // kernel (deterministic), then an Adam step on FP32 master weights.
 #include "gp_nn_internal.h"
 
@@ -470,19 +470,35 @@ __global__ void __launch_bounds__(256, 1) nn_train_kernel(NNParams P, NNTrain T)
     wgrad(s.x, LDX, s.d1, 0, warp, 1, part + kOffW0);
 }
 
-// grad[q] = sum over blocks of partial[b][q], in block order; loss likewise.
-__global__ void nn_reduce_kernel(const float *partials, int blocks, float *grad, const float *loss_partials,
-                                 float *loss) {
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
+// grad[q] = sum over blocks of partial[b][q]; loss likewise.  A block sums 32
+// parameters: warp g adds the g-th eighth of the partials in order, then the
+// eight sums are added in order (fixed grouping, so the result does not
+// depend on timing).  One thread per parameter over all partials left 37
+// blocks waiting on a chain of 256 additions each.
+constexpr int kReduceWarps = 8;
+__global__ void __launch_bounds__(32 * kReduceWarps) nn_reduce_kernel(const float *partials, int blocks, float *grad,
+                                                                      const float *loss_partials, float *loss) {
+    __shared__ float part[kReduceWarps][32];
+    const int lane = threadIdx.x & 31, g = threadIdx.x >> 5, q = blockIdx.x * 32 + lane;
+    const int per = (blocks + kReduceWarps - 1) / kReduceWarps, b0 = g * per, b1 = min(blocks, b0 + per);
+    float v = 0.f;
     if (q < kNNParams) {
-        float v = 0.f;
-        for (int b = 0; b < blocks; ++b) v += partials[(size_t)b * kNNParams + q];
-        grad[q] = v;
+#pragma unroll 8
+        for (int b = b0; b < b1; ++b) v += partials[(size_t)b * kNNParams + q];
     }
-    if (q == 0) {
-        float v = 0.f;
-        for (int b = 0; b < blocks; ++b) v += loss_partials[b];
-        *loss = v;
+    part[g][lane] = v;
+    __syncthreads();
+    if (g == 0 && q < kNNParams) {
+        float s = 0.f;
+        for (int w = 0; w < kReduceWarps; ++w) s += part[w][lane];
+        grad[q] = s;
+    }
+    if (blockIdx.x == 0 && g == 1) {
+        float l = 0.f;
+        for (int b = lane; b < blocks; b += 32) l += loss_partials[b];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+        if (lane == 0) *loss = l;
     }
 }
 
@@ -522,7 +538,7 @@ cudaError_t nn_launch_train(const NNParams &P, const NNTrain &T, int blocks, cud
     nn_train_kernel<<<blocks, 256, sizeof(TrainSmem), s>>>(P, T);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    nn_reduce_kernel<<<(kNNParams + 255) / 256, 256, 0, s>>>(T.partials, blocks, T.grad, T.loss_partials, T.loss);
+    nn_reduce_kernel<<<(kNNParams + 31) / 32, 32 * kReduceWarps, 0, s>>>(T.partials, blocks, T.grad, T.loss_partials, T.loss);
     return cudaGetLastError();
 }
 
