@@ -251,9 +251,12 @@ gp_status gp_set_stream(gp_handle h, void *cuda_stream);
 gp_status gp_sync(gp_handle h);
 
 /* Window of the windowed back substitution per axis for imaginary (mode 0)
- * or real (mode 1) time; 0 means the exact two-pass solve is used.  By
- * default FP32 fields use the smallest admissible window and FP64 fields the
- * exact solve (FP64 arithmetic, not memory, bounds the FP64 forms). */
+ * or real (mode 1) time; 0 means an exact solve is used.  By default FP32
+ * fields use the smallest admissible window and FP64 fields the exact solve
+ * (FP64 arithmetic, not memory, bounds the FP64 forms): two passes with one
+ * thread per line, or, on grids with too few lines to fill the GPU that way,
+ * cyclic reduction to below a quarter of the unit roundoff.  A window, a
+ * segment length or a block size set for an axis keeps the two-pass form. */
 gp_status gp_get_window(gp_handle h, int mode, int window[3]);
 
 /* Override the window of every axis and mode: -1 restores the automatic
@@ -322,7 +325,7 @@ gp_status gp_set_tma_lines(gp_handle h, int axes);
 gp_status gp_get_tma_lines(gp_handle h, int *axes);
 
 /* Threads per block of the line-solve kernel of one axis (multiple of 32,
- * 32..256). */
+ * 32..256; until set: 64, or 32 on x and y for the exact two-pass form). */
 gp_status gp_set_threads(gp_handle h, int axis, int threads);
 
 /* Interior nodes per segment of the line solves of one axis (0 = the
@@ -336,7 +339,8 @@ gp_status gp_get_segments(gp_handle h, int mode, int seg_len[3], int n_seg[3]);
 
 /* Autotuner: for each axis, time the line-solve kernel of the imaginary-
  * (realtime = 0) or real-time (1) step on this handle's grid under every
- * candidate launch setting -- threads per block (64, 128), segment length
+ * candidate launch setting -- threads per block (64, 128; for exact solves
+ * also 32 and the automatic form), segment length
  * (automatic, 64, 128, 256, whole line) and one or two lines per thread --
  * with CUDA events over `reps` launches after a warm-up, and keep the
  * fastest.  psi is left unchanged (the trials run on a copy).  Choices are
@@ -480,11 +484,13 @@ gp_status gp_batch_set_segments(gp_batch b, int seg_len);
 /* Steps per CUDA graph (default 16; 0 or 1: launch by launch). */
 gp_status gp_batch_set_graph_block(gp_batch b, int steps);
 /* Stream groups of a batched step (1..16, default 2): the active instances
- * are split into groups balanced by sites, and each group's x, y and z
- * sweeps run as one chain of launches on a stream of its own, forked from
- * and joined back into the batch's stream (and captured into its graphs as
- * parallel branches), so launches of different groups overlap.  psi is the
- * same for every setting. */
+ * are split into groups by the launches they take (line groups on x and y,
+ * the z sweep's form; with more than one group asked for, every such kind has
+ * at least one) and balanced by sites, and each group's x, y and z sweeps run
+ * as one chain of launches on a stream of its own, forked from and joined
+ * back into the batch's stream (and captured into its graphs as parallel
+ * branches), so launches of different groups overlap.  psi is the same for
+ * every setting. */
 gp_status gp_batch_set_streams(gp_batch b, int streams);
 /* z sweep of the instances whose rows fit the TMA form (the rules of
  * gp_set_tma, at the batch's z window; at most 64 instances, the first ones
