@@ -139,6 +139,9 @@ bool choose_pcr(long long lines, int n, Form form, Kind kind, int levels, int el
 void append_tables(const Geometry &G, bool f32, int modes, std::vector<char> &host, Tables &T, PcrTables pcr) {
     const size_t rsz = f32 ? sizeof(float) : sizeof(double);
     const double eps = f32 ? std::ldexp(1.0, -24) : std::ldexp(1.0, -53);
+    // nothing of an earlier dt stays: an axis that takes the cyclic reduction
+    // at one dt and not at the next has no levels and no table offsets
+    T = Tables();
     size_t off = align_up(host.size(), 256);
     for (int mode = 0; mode < modes; ++mode) {
         for (int ax = 0; ax < 3; ++ax) {

@@ -1,0 +1,37 @@
+"""The host rules that choose kernels and lay out their tables, asked of
+libgpcn.so itself through a small C++ client (no GPU)."""
+import os
+import subprocess
+
+import pytest
+
+from paper_1601_04641_gb300 import _native as N
+from paper_1601_04641_gb300 import build
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def probe(tmp_path_factory):
+    build.build()
+    exe = str(tmp_path_factory.mktemp("probe") / "probe")
+    cuda = os.path.join(os.path.dirname(os.path.dirname(build.nvcc())), "include")
+    lib = os.path.dirname(N.LIB_PATH)
+    subprocess.run(["g++", "-std=c++17", "-I", build.INCLUDE, "-I", build.CSRC, "-I", cuda, os.path.join(HERE, "host_probe.cpp"),
+                    "-L", lib, "-lgpcn", "-Wl,-rpath," + lib, "-o", exe], check=True, capture_output=True, text=True)
+
+    def ask(*args):
+        out = subprocess.run([exe] + [str(a) for a in args], check=True, capture_output=True, text=True, timeout=120).stdout
+        return [[float(v) for v in line.split()] for line in out.splitlines()]
+
+    return ask
+
+
+@pytest.mark.parametrize("shape,modes,factors", [
+    ((96, 96, 96), 1, (0.1, 0.5, 0.1, 1.0, 0.1)), ((100, 100, 100), 1, (0.1, 0.5, 0.1)), ((80, 80, 80), 2, (0.05, 1.0, 0.05)),
+    ((64, 48, 40), 1, (0.1, 1.0, 10.0, 0.1)), ((160, 128, 96), 2, (0.02, 0.1, 1.0))])
+def test_tables_of_a_new_dt_keep_nothing_of_the_old(probe, shape, modes, factors):
+    """A handle's tables are rebuilt in place when dt changes: an axis that takes the cyclic reduction at one dt and not at
+    the next must not keep the old levels and offsets."""
+    got = probe("tables", *shape, modes, *factors)
+    assert [g[0] for g in got] == [1.0] * len(factors)
