@@ -213,13 +213,38 @@ Geometry geom(gp_handle h) {
     return G;
 }
 
-// Build and upload the coefficient tables of both modes and all axes, and
-// pick the window of the windowed backward sweep for each.
-gp_status build_coefficients(gp_handle h) {
+// Build and upload the coefficient tables of both modes and all axes for a
+// time step, and pick the window of the windowed backward sweep for each.
+// Which tables there are depends on dt (the cyclic reduction's), so a new dt
+// may need a larger buffer: it is allocated before the old one is given up,
+// and a failure leaves the handle at its old dt.
+gp_status build_coefficients(gp_handle h, double dt) {
     const bool f32 = h->prec != GP_F64;  // FP32 tables for FP32 arithmetic (FP32 and FP16 storage)
+    Geometry G = geom(h);
+    G.dt = dt;
+    Tables tab;
     std::vector<char> host;
-    append_tables(geom(h), f32, modes_of(h), host, h->tab, kPcrChosen);
+    append_tables(G, f32, modes_of(h), host, tab, kPcrChosen);
     const size_t off = host.size();
+    char *dst = h->d_coef;
+    if (h->coef_bytes < off && gpcn::dev_malloc(&dst, off) != cudaSuccess) {
+        cudaGetLastError();
+        return fail(h, GP_ERR_NOMEM, "cudaMalloc of the coefficient tables failed");
+    }
+    cudaError_t e = cudaMemcpyAsync(dst, host.data(), off, cudaMemcpyHostToDevice, h->stream);
+    const cudaError_t es = cudaStreamSynchronize(h->stream);
+    if (e == cudaSuccess) e = es;
+    if (e != cudaSuccess) {
+        if (dst != h->d_coef) cudaFree(dst);
+        return fail(h, GP_ERR_CUDA, std::string("copy of the coefficient tables: ") + cudaGetErrorString(e));
+    }
+    if (dst != h->d_coef) {
+        cudaFree(h->d_coef);
+        h->d_coef = dst;
+        h->coef_bytes = off;
+    }
+    h->dt = dt;
+    h->tab = tab;
     for (int mode = 0; mode < modes_of(h); ++mode)
         for (int ax = 0; ax < 3; ++ax) {
             const AxisTables &at = h->tab.ax[mode][ax];
@@ -230,19 +255,6 @@ gp_status build_coefficients(gp_handle h) {
             h->window[mode][ax] = w;
         }
     for (bool &set : h->axis_window) set = false;
-    if (h->d_coef && h->coef_bytes < off) {
-        cudaFree(h->d_coef);
-        h->d_coef = nullptr;
-    }
-    if (!h->d_coef) {
-        if (gpcn::dev_malloc(&h->d_coef, off) != cudaSuccess) {
-            cudaGetLastError();
-            return fail(h, GP_ERR_NOMEM, "cudaMalloc of the coefficient tables failed");
-        }
-        h->coef_bytes = off;
-    }
-    GP_CK(h, cudaMemcpyAsync(h->d_coef, host.data(), off, cudaMemcpyHostToDevice, h->stream));
-    GP_CK(h, cudaStreamSynchronize(h->stream));
     return GP_OK;
 }
 
@@ -358,7 +370,7 @@ gp_status create_common(gp_handle *out, gp_grid grid, double dt, double gamma, d
         return fail(nullptr, GP_ERR_NOMEM, "cudaMalloc of the second psi buffer failed");
     }
     st = alloc_scratch(h);
-    if (st == GP_OK) st = build_coefficients(h);
+    if (st == GP_OK) st = build_coefficients(h, dt);
     {
         const long long rows = (long long)grid.nx * grid.ny;
         h->zmap_ok = encode_z_map(&h->zmap[0], h->buf[0], grid.nz, rows, (int)h->elem) &&
@@ -804,8 +816,7 @@ gp_status gp_set_dt(gp_handle h, double dt) {
     if (!finite_pos(dt)) return fail(h, GP_ERR_ARG, "dt must be finite and > 0");
     if ((st = settle(h)) != GP_OK) return st;  // the pending half kick belongs to the old dt
     drop_graphs(h);
-    h->dt = dt;
-    return build_coefficients(h);
+    return build_coefficients(h, dt);
 }
 
 gp_status gp_step_imag(gp_handle h, int nsteps) {
