@@ -53,7 +53,11 @@ __device__ __forceinline__ void mbar_arrive(unsigned bar) {
 }
 // Programmatic dependent launch: let the next launch of the stream begin, and
 // wait until the previous one has completed and its writes are visible
-// (nothing to wait for in a launch without the attribute).
+// (nothing to wait for in a launch without the attribute).  What the previous
+// launch writes (psi, the renormalisation factor) is read by ordinary loads
+// after the wait; __ldg is for tables alone: its non-coherent load is defined
+// only where nobody writes during the whole life of the kernel, which here
+// begins before the previous launch has ended.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 

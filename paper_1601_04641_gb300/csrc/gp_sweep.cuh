@@ -1158,7 +1158,7 @@ __device__ __forceinline__ void solve_line_exact(int n, int tconst, R kap, const
 template <typename R, int KIND> __device__ __forceinline__ void kick_init(KickState<R> &k, const SweepArgs &a,
                                                                           long long L) {
     const int j = (int)(L / a.nz), kk = (int)(L % a.nz);
-    k.s = (R)__ldg(a.scale);
+    k.s = (R)*a.scale;  // not through __ldg: under a dependent launch the previous sweep writes it while this kernel lives
     k.dtg = (R)(a.dt * a.g);
     k.ex = static_cast<const R *>(a.kick_ex);
     if (a.kick_ex) {
