@@ -24,6 +24,7 @@
 #include "gp.h"
 #include "gp_host.h"
 #include "gp_internal.h"
+#include "gp_optin.h"
 
 #include <algorithm>
 #include <cmath>
@@ -506,13 +507,9 @@ template <typename R, bool CPLX> cudaError_t radial_launch(const AxArgs &args, c
     const size_t line = 2 * (size_t)(args.nx - 2) * sizeof(typename AxElem<R, CPLX>::V);
     const int tl = (int)std::min<size_t>(std::min<size_t>(32, (args.nz + 151) / 152), kPcrSmem / line);
     if (tl > 0) {
-        static bool attr = false;  // opt in once to more than 48 KB of dynamic shared memory
-        if (!attr) {
-            cudaError_t e = cudaFuncSetAttribute(axial_radial_smem_kernel<R, CPLX>,
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPcrSmem);
-            if (e != cudaSuccess) return e;
-            attr = true;
-        }
+        static SmemOptIn kept;
+        const cudaError_t e = opt_in_smem(kept, axial_radial_smem_kernel<R, CPLX>, kPcrSmem);
+        if (e != cudaSuccess) return e;
         axial_radial_smem_kernel<R, CPLX><<<(args.nz + tl - 1) / tl, kRadialThreads, tl * line, s>>>(args, tl);
         return cudaGetLastError();
     }

@@ -24,6 +24,7 @@
 #pragma once
 
 #include "gp_async.cuh"
+#include "gp_optin.h"
 #include "gp_sweep.cuh"
 
 namespace gpcn {
@@ -198,13 +199,9 @@ __global__ void __launch_bounds__(1024) lines_pcr_kernel(SweepArgs a, PcrArgs p)
 template <class F, int KIND, bool RADIAL, int NS>
 inline cudaError_t launch_pcr_ns(const SweepArgs &a, const PcrArgs &p, int threads, size_t smem, cudaStream_t s) {
     const unsigned grid = (unsigned)((a.n_lines + p.tl - 1) / p.tl);
-    static bool attr = false;  // opt in once to more than 48 KB of dynamic shared memory
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(lines_pcr_kernel<F, KIND, RADIAL, NS>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPcrSmem);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    static SmemOptIn kept;
+    const cudaError_t e = opt_in_smem(kept, lines_pcr_kernel<F, KIND, RADIAL, NS>, kPcrSmem);
+    if (e != cudaSuccess) return e;
     if (p.dependent) return launch_dependent(lines_pcr_kernel<F, KIND, RADIAL, NS>, grid, threads, smem, s, a, p);
     lines_pcr_kernel<F, KIND, RADIAL, NS><<<grid, threads, smem, s>>>(a, p);
     return cudaGetLastError();

@@ -16,6 +16,7 @@
 // written as per-block partial gradients, summed in a fixed grouping by a second
 // kernel (deterministic), then an Adam step on FP32 master weights.
 #include "gp_nn_internal.h"
+#include "gp_optin.h"
 
 #include <cuda_bf16.h>
 
@@ -528,15 +529,11 @@ __global__ void nn_deploy_kernel(NNParams P) {
 size_t nn_train_smem() { return sizeof(TrainSmem); }
 
 cudaError_t nn_launch_train(const NNParams &P, const NNTrain &T, int blocks, cudaStream_t s) {
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(nn_train_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)sizeof(TrainSmem));
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    static SmemOptIn kept;
+    cudaError_t e = opt_in_smem(kept, nn_train_kernel, sizeof(TrainSmem));
+    if (e != cudaSuccess) return e;
     nn_train_kernel<<<blocks, 256, sizeof(TrainSmem), s>>>(P, T);
-    cudaError_t e = cudaGetLastError();
+    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     nn_reduce_kernel<<<(kNNParams + 31) / 32, 32 * kReduceWarps, 0, s>>>(T.partials, blocks, T.grad, T.loss_partials, T.loss);
     return cudaGetLastError();

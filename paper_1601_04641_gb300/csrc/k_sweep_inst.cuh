@@ -2,6 +2,7 @@
 // form and precision and dispatches a launch to them.
 #pragma once
 
+#include "gp_optin.h"
 #include "gp_sweep.cuh"
 #include "gp_sweep_tma.cuh"
 
@@ -13,13 +14,9 @@ static cudaError_t launch_contig_w(const SweepArgs &a, cudaStream_t s) {
     const unsigned threads = 32 * kTileWarps;
     const dim3 grid((unsigned)((a.n_lines + threads - 1) / threads), (unsigned)a.n_seg);
     const size_t smem = kTileWarps * tile_warp_bytes<V, W>();
-    static bool attr = false;  // opt in once to more than 48 KB of dynamic shared memory
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(sweep_contig_kernel<F, R, W>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    static SmemOptIn kept;
+    const cudaError_t e = opt_in_smem(kept, sweep_contig_kernel<F, R, W>, smem);
+    if (e != cudaSuccess) return e;
     sweep_contig_kernel<F, R, W><<<grid, threads, smem, s>>>(a);
     return cudaGetLastError();
 }
@@ -30,13 +27,9 @@ static cudaError_t launch_tma_w(const SweepArgs &a, const TmaMaps &m, cudaStream
         const long long rows = (long long)kTmaWarps * kTmaRows;
         const unsigned grid = (unsigned)((a.n_lines + rows - 1) / rows);
         constexpr size_t smem = tma_smem_bytes<store_t<F>, W>();
-        static bool attr = false;  // opt in once to more than 48 KB of dynamic shared memory
-        if (!attr) {
-            cudaError_t e = cudaFuncSetAttribute(sweep_tma_kernel<F, R, W>,
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-            attr = true;
-        }
+        static SmemOptIn kept;
+        const cudaError_t e = opt_in_smem(kept, sweep_tma_kernel<F, R, W>, smem);
+        if (e != cudaSuccess) return e;
         sweep_tma_kernel<F, R, W><<<grid, kTmaWarps * 32, smem, s>>>(a, m);
         return cudaGetLastError();
     } else {
@@ -73,13 +66,9 @@ static cudaError_t launch_lines_tma_wl(const SweepArgs &a, const TmaMaps &m, cud
     const long long warps = (a.n_lines / a.inner) * wpr;
     const dim3 grid((unsigned)((warps + kLineTmaWarps - 1) / kLineTmaWarps), (unsigned)a.n_seg);
     constexpr size_t smem = line_tma_smem<MV>();
-    static bool attr = false;  // opt in once to more than 48 KB of dynamic shared memory
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(sweep_lines_tma_kernel<F, R, W, KIND, LPT>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    static SmemOptIn kept;
+    const cudaError_t e = opt_in_smem(kept, sweep_lines_tma_kernel<F, R, W, KIND, LPT>, smem);
+    if (e != cudaSuccess) return e;
     sweep_lines_tma_kernel<F, R, W, KIND, LPT><<<grid, kLineTmaWarps * 32, smem, s>>>(a, m);
     return cudaGetLastError();
 }
@@ -103,12 +92,10 @@ static cudaError_t launch_lines_wl_any(const SweepLaunch &L, const SweepArgs &a,
             return cudaGetLastError();
         }
     }
-    static int attr = 0;  // largest dynamic shared memory opted in so far
-    if ((int)smem > attr && smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(sweep_lines_kernel<F, R, W, KIND, LPT, 0>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    static SmemOptIn kept;
+    if (smem > 48 * 1024) {
+        const cudaError_t e = opt_in_smem(kept, sweep_lines_kernel<F, R, W, KIND, LPT, 0>, smem);
         if (e != cudaSuccess) return e;
-        attr = (int)smem;
     }
     sweep_lines_kernel<F, R, W, KIND, LPT, 0><<<grid, threads, smem, s>>>(a);
     return cudaGetLastError();
@@ -153,12 +140,10 @@ static cudaError_t launch_batch_lines_wl(const BatchLaunch &b, cudaStream_t s) {
     using V = typename LinesPerThread<F, LPT>::M::MemV;
     const unsigned threads = kBatchLineThreads;
     const size_t smem = W > 0 ? column_ring_bytes<V, W>(threads) : 0;
-    static bool attr = false;
-    if (!attr && smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(batch_lines_kernel<F, R, W, KIND, LPT>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    static SmemOptIn kept;
+    if (smem > 48 * 1024) {
+        const cudaError_t e = opt_in_smem(kept, batch_lines_kernel<F, R, W, KIND, LPT>, smem);
         if (e != cudaSuccess) return e;
-        attr = true;
     }
     BatchDesc d{b.args, b.first, b.gridx, b.n};
     batch_lines_kernel<F, R, W, KIND, LPT><<<b.total_blocks, threads, smem, s>>>(d);
@@ -183,13 +168,9 @@ template <class F, typename R, int W>
 static cudaError_t launch_batch_contig_w(const BatchLaunch &b, cudaStream_t s) {
     using V = typename F::V;
     const size_t smem = kTileWarps * tile_warp_bytes<V, W>();
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(batch_contig_kernel<F, R, W>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    static SmemOptIn kept;
+    const cudaError_t e = opt_in_smem(kept, batch_contig_kernel<F, R, W>, smem);
+    if (e != cudaSuccess) return e;
     BatchDesc d{b.args, b.first, b.gridx, b.n};
     batch_contig_kernel<F, R, W><<<b.total_blocks, 32 * kTileWarps, smem, s>>>(d);
     return cudaGetLastError();
@@ -202,13 +183,9 @@ static cudaError_t launch_batch_tma_w(const BatchLaunch &b, cudaStream_t s) {
     if constexpr (tma_supported<F, W>()) {
         if (b.n > kTmaBatch) return cudaErrorInvalidValue;
         constexpr size_t smem = tma_smem_bytes<typename F::V, W>();
-        static bool attr = false;
-        if (!attr) {
-            cudaError_t e = cudaFuncSetAttribute(batch_tma_kernel<F, R, W>,
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-            attr = true;
-        }
+        static SmemOptIn kept;
+        const cudaError_t e = opt_in_smem(kept, batch_tma_kernel<F, R, W>, smem);
+        if (e != cudaSuccess) return e;
         BatchDesc d{b.args, b.first, b.gridx, b.n};
         batch_tma_kernel<F, R, W><<<b.total_blocks, kTmaWarps * 32, smem, s>>>(d, *b.tma);
         return cudaGetLastError();

@@ -1,10 +1,14 @@
 // Asks libgpcn.so's host side (no GPU) what it would do; see test_host_rules.py.
+//   optin                             the calls a kernel's opt-in makes: per device, per growth, on failure, from threads
 //   tables NX NY NZ MODES DT DT ...   tables built for each dt in turn into one Tables, against fresh ones: 1 where equal
 #include "gp_host.h"
+#include "gp_optin.h"
 
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <thread>
+#include <vector>
 
 using namespace gpcn;
 
@@ -13,7 +17,46 @@ static bool same(const AxisTables &a, const AxisTables &b) {
            a.pcr_levels == b.pcr_levels && a.off_pcr == b.off_pcr && a.off_pcr_inv == b.off_pcr_inv && a.cp_max == b.cp_max;
 }
 
+// Bytes set on a device by a sequence of raises, as cudaFuncSetAttribute would see them.
+static int optin() {
+    SmemOptIn kept;
+    int limit[3] = {0, 0, 0}, calls[3] = {0, 0, 0};
+    auto raise = [&](int dev, int bytes) {
+        return kept.raise(dev, bytes, [&](int b) {
+            ++calls[dev];
+            limit[dev] = b;
+            return cudaSuccess;
+        });
+    };
+    for (int dev : {0, 1, 0, 1, 2}) raise(dev, 60000);
+    raise(1, 70000);
+    raise(1, 50000);
+    for (int dev = 0; dev < 3; ++dev) std::printf("%d %d\n", limit[dev], calls[dev]);
+    // a failed set is not remembered
+    SmemOptIn bad;
+    int tries = 0;
+    for (int q = 0; q < 2; ++q) bad.raise(0, 60000, [&](int) { ++tries; return cudaErrorInvalidValue; });
+    std::printf("%d %d\n", tries, (int)bad.raise(kOptInDevices, 1, [&](int) { ++tries; return cudaSuccess; }));
+    // threads of different sizes: never lowered
+    SmemOptIn shared;
+    int high = 0, lowered = 0;
+    std::vector<std::thread> threads;
+    for (int t = 0; t < 8; ++t)
+        threads.emplace_back([&, t] {
+            for (int q = 0; q < 1000; ++q)
+                shared.raise(0, 50000 + (q * 37 + t * 911) % 50000, [&](int b) {  // under the lock
+                    lowered += b < high;
+                    high = b;
+                    return cudaSuccess;
+                });
+        });
+    for (auto &t : threads) t.join();
+    std::printf("%d %d\n", high, lowered);
+    return 0;
+}
+
 int main(int argc, char **argv) {
+    if (argc > 1 && !std::strcmp(argv[1], "optin")) return optin();
     if (argc > 6 && !std::strcmp(argv[1], "tables")) {
         Geometry G;
         for (int q = 0; q < 3; ++q) {

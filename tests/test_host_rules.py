@@ -1,6 +1,7 @@
 """The host rules that choose kernels and lay out their tables, asked of
 libgpcn.so itself through a small C++ client (no GPU)."""
 import os
+import re
 import subprocess
 
 import pytest
@@ -17,7 +18,7 @@ def probe(tmp_path_factory):
     exe = str(tmp_path_factory.mktemp("probe") / "probe")
     cuda = os.path.join(os.path.dirname(os.path.dirname(build.nvcc())), "include")
     lib = os.path.dirname(N.LIB_PATH)
-    subprocess.run(["g++", "-std=c++17", "-I", build.INCLUDE, "-I", build.CSRC, "-I", cuda, os.path.join(HERE, "host_probe.cpp"),
+    subprocess.run(["g++", "-std=c++17", "-pthread", "-I", build.INCLUDE, "-I", build.CSRC, "-I", cuda, os.path.join(HERE, "host_probe.cpp"),
                     "-L", lib, "-lgpcn", "-Wl,-rpath," + lib, "-o", exe], check=True, capture_output=True, text=True)
 
     def ask(*args):
@@ -35,3 +36,18 @@ def test_tables_of_a_new_dt_keep_nothing_of_the_old(probe, shape, modes, factors
     the next must not keep the old levels and offsets."""
     got = probe("tables", *shape, modes, *factors)
     assert [g[0] for g in got] == [1.0] * len(factors)
+
+
+def test_shared_memory_opt_in_is_kept_per_device(probe):
+    """The limit is a property of a kernel on one device: the second device gets its own call, a larger launch raises it, a
+    smaller one and one from another thread never lower it, and a failed call is made again."""
+    d0, d1, d2, bad, threads = probe("optin")
+    assert d0 == [60000, 1] and d1 == [70000, 2] and d2 == [60000, 1]
+    assert bad == [2, 0]
+    assert threads[0] == 50000 + 999 * 37 + 7 * 911 and threads[1] == 0
+
+
+def test_no_launcher_keeps_a_process_wide_opt_in():
+    for name in sorted(os.listdir(build.CSRC)):
+        src = open(os.path.join(build.CSRC, name)).read()
+        assert not re.search(r"static\s+(bool|int)\s+attr\b", src), name
