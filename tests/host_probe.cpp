@@ -36,7 +36,8 @@ static int optin() {
     SmemOptIn bad;
     int tries = 0;
     for (int q = 0; q < 2; ++q) bad.raise(0, 60000, [&](int) { ++tries; return cudaErrorInvalidValue; });
-    std::printf("%d %d\n", tries, (int)bad.raise(kOptInDevices, 1, [&](int) { ++tries; return cudaSuccess; }));
+    const int beyond = (int)bad.raise(kOptInDevices, 1, [&](int) { ++tries; return cudaSuccess; });
+    std::printf("%d %d\n", tries, beyond);
     // threads of different sizes: never lowered
     SmemOptIn shared;
     int high = 0, lowered = 0;
