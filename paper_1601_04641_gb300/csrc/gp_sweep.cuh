@@ -79,11 +79,7 @@ __device__ __forceinline__ void g_sincos(double x, double *s, double *c) { sinco
 //         |y| <= 0.05 (next term below 2^-27 of exp(-y)).
 //   FP64: sin through x^9, cos through x^10 for |x| <= 0.1 (next terms below
 //         2^-58 relative); exp(-y) - 1 through y^7 for |y| <= 0.02 (next
-//         term below 2^-60 of exp(-y)).  Groups of phases within 0.03 (the
-//         phases of a real-time step at dt = 0.02 d^2) take sin through x^7
-//         and cos through x^6 (next terms below 2^-58 and 2^-55): the FP64
-//         forms are bound by the FP64 pipe (2 lanes a clock and SM), and
-//         this saves 3 of the kick's operations.
+//         term below 2^-60 of exp(-y)).
 // Imaginary-time factors are formed as deviations from one (exp(-y) - 1,
 // and the trap tables hold exp(-dt V_a) - 1): a factor rounded once near one
 // and applied at every step acts as a potential error of u / dt (u the unit
@@ -92,7 +88,7 @@ __device__ __forceinline__ void g_sincos(double x, double *s, double *c) { sinco
 // rounded once is off by u |dt V|, a potential error of u |V|.
 template <typename R> struct Series;
 template <> struct Series<float> {
-    static constexpr float kTrig = 0.2f, kExp = 0.05f, kTrigNear = 0.f;  // no nearer tier
+    static constexpr float kTrig = 0.2f, kExp = 0.05f;
     __device__ __forceinline__ static void sincos(float x, float *sn, float *cs) {
         const float x2 = x * x;
         *sn = x * fmaf(x2, fmaf(x2, 1.f / 120.f, -1.f / 6.f), 1.f);
@@ -103,12 +99,7 @@ template <> struct Series<float> {
     }
 };
 template <> struct Series<double> {
-    static constexpr double kTrig = 0.1, kExp = 0.02, kTrigNear = 0.03;
-    __device__ __forceinline__ static void sincos_near(double x, double *sn, double *cs) {  // |x| <= kTrigNear
-        const double x2 = x * x;
-        *sn = x * fma(x2, fma(x2, fma(x2, -1.0 / 5040.0, 1.0 / 120.0), -1.0 / 6.0), 1.0);
-        *cs = fma(x2, fma(x2, fma(x2, -1.0 / 720.0, 1.0 / 24.0), -0.5), 1.0);
-    }
+    static constexpr double kTrig = 0.1, kExp = 0.02;
     __device__ __forceinline__ static void sincos(double x, double *sn, double *cs) {
         const double x2 = x * x;
         *sn = x * fma(x2, fma(x2, fma(x2, fma(x2, 1.0 / 362880.0, -1.0 / 5040.0), 1.0 / 120.0),
@@ -387,7 +378,7 @@ template <typename R> struct FRealTime : LineForm<cx<R>> {
             constexpr int G = NB < kKickGroup ? NB : kKickGroup;
             R px[G], th[G];
             V q[G];
-            bool small = true, near = Series<R>::kTrigNear > R(0);
+            bool small = true;
 #pragma unroll
             for (int i = 0; i < G; ++i) px[i] = __ldg(k.px + node0 + g0 + i);
 #pragma unroll
@@ -400,18 +391,6 @@ template <typename R> struct FRealTime : LineForm<cx<R>> {
             for (int i = 0; i < G; ++i) {
                 th[i] = fma(k.dtg, abs2(q[i]), px[i] + k.pyz);
                 small = small && fabs(th[i]) <= Series<R>::kTrig;
-                near = near && fabs(th[i]) <= Series<R>::kTrigNear;
-            }
-            if constexpr (sizeof(R) == 8) {
-                if (near) {
-#pragma unroll
-                    for (int i = 0; i < G; ++i) {
-                        R sn, cs;
-                        Series<R>::sincos_near(th[i], &sn, &cs);
-                        v[g0 + i] = V{fma(cs, q[i].re, sn * q[i].im), fma(cs, q[i].im, -sn * q[i].re)};
-                    }
-                    continue;
-                }
             }
             if (small) {
 #pragma unroll
