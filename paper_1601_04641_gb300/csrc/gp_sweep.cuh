@@ -143,25 +143,13 @@ template <typename R> __device__ __forceinline__ R kick_dev(R ex, R eyz, R m) {
     return fma(t, m, t + m);
 }
 
-// q (1 + ex)(1 + eyz)(1 + m).  FP64 applies the three deviations one after
-// the other: three operations on the FP64 pipe instead of five, each rounded
-// at the unit roundoff of the value.
-template <typename R> __device__ __forceinline__ R kick_apply(R q, R ex, R eyz, R m) {
-    if constexpr (sizeof(R) == 8) {
-        q = fma(q, ex, q);
-        q = fma(q, eyz, q);
-        return fma(q, m, q);
-    } else {
-        return fma(q, kick_dev(ex, eyz, m), q);
-    }
-}
-// The same with m = exp(-y) - 1 of any size; FP64 beyond the series
-// multiplies by exp(-y) itself, which does not vanish where m rounds to -1.
-template <typename R> __device__ __forceinline__ R kick_apply_full(R q, R ex, R eyz, R y) {
-    if constexpr (sizeof(R) == 8) {
-        if (fabs(y) > Series<R>::kExp) return fma(fma(q, ex, q), eyz, fma(q, ex, q)) * exp_full(-y);
-    }
-    return kick_apply(q, ex, eyz, kick_expm1m(y));
+// FP64 where the nonlinear factor has fallen below a half (y > ln 2): there m
+// nears -1 and 1 + m loses the factor's last bits, all of them by y = 37 (a
+// three-node field with dt g |psi|^2 = 315 came out empty), so the value is
+// multiplied by exp(-y) itself.  Nearer one the deviation is the more exact.
+template <typename R> __device__ __forceinline__ bool kick_fades(R y) { return sizeof(R) == 8 && y > R(0.6931471805599453); }
+template <typename R> __device__ __forceinline__ R kick_faded(R q, R ex, R eyz, R e) {  // e = exp(-y)
+    return fma(q, fma(ex, eyz, ex + eyz), q) * e;
 }
 
 // Per-site kick state of one x line.  Imaginary time: exp(-dt V) is the
@@ -239,7 +227,9 @@ template <typename R> struct FImagReal : LineForm<R> {
     __device__ __forceinline__ static R abs2(V v) { return v * v; }
     __device__ __forceinline__ static V kick(V p, const KickState<R> &k, int node) {
         const V q = p * k.s;
-        return kick_apply_full(q, __ldg(k.ex + node), k.eyz, k.dtg * (q * q));
+        const R ex = __ldg(k.ex + node), y = k.dtg * (q * q);
+        if (kick_fades(y)) return kick_faded(q, ex, k.eyz, (R)exp_full(-y));
+        return fma(q, kick_dev(ex, k.eyz, kick_expm1m(y)), q);
     }
     // kick of NB consecutive nodes from node0: table loads issued together,
     // one series-range test per group, values equal kick's
@@ -260,7 +250,7 @@ template <typename R> struct FImagReal : LineForm<R> {
             }
             if (small) {
 #pragma unroll
-                for (int i = 0; i < G; ++i) v[g0 + i] = kick_apply(q[i], ex[i], k.eyz, Series<R>::expm1m(y[i]));
+                for (int i = 0; i < G; ++i) v[g0 + i] = fma(q[i], kick_dev(ex[i], k.eyz, Series<R>::expm1m(y[i])), q[i]);
             } else {
 #pragma unroll
                 for (int i = 0; i < G; ++i) v[g0 + i] = kick(v[g0 + i], k, node0 + g0 + i);
@@ -294,13 +284,13 @@ template <typename R> struct FImagCplx : LineForm<cx<R>> {
     __device__ __forceinline__ static R abs2(V v) { return fma(v.re, v.re, v.im * v.im); }
     __device__ __forceinline__ static V kick(V p, const KickState<R> &k, int node) {
         const V q{p.re * k.s, p.im * k.s};
-        const R y = k.dtg * abs2(q), ex = __ldg(k.ex + node);
-        if constexpr (sizeof(R) == 8) {
-            return V{kick_apply_full(q.re, ex, k.eyz, y), kick_apply_full(q.im, ex, k.eyz, y)};
-        } else {
-            const R f = kick_dev(ex, k.eyz, kick_expm1m(y));
-            return V{fma(q.re, f, q.re), fma(q.im, f, q.im)};
+        const R ex = __ldg(k.ex + node), y = k.dtg * abs2(q);
+        if (kick_fades(y)) {
+            const R e = (R)exp_full(-y);
+            return V{kick_faded(q.re, ex, k.eyz, e), kick_faded(q.im, ex, k.eyz, e)};
         }
+        const R f = kick_dev(ex, k.eyz, kick_expm1m(y));
+        return V{fma(q.re, f, q.re), fma(q.im, f, q.im)};
     }
     static constexpr bool kChunkKick = true;
     template <int NB> __device__ __forceinline__ static void kick_chunk(V (&v)[NB], const KickState<R> &k, int node0) {

@@ -4,7 +4,13 @@ the buffer after one step (without its renormalisation factor) holds the
 kicked values.
 
 A node's kick is a function of its own value: the same whatever its
-neighbours hold, however its line is cut into chunks, and in both solves."""
+neighbours hold, however its line is cut into chunks, and in both solves.
+
+Error bounds, u = 2^-53.  Imaginary time at small exponents: the factor's
+deviation from one is a sum of four terms, each within 8 relative roundings,
+and the value is rounded once: u (1 + 8 sum|dev|) of the result.  At large
+exponents: the exponent is within 3 relative roundings, the product within 6:
+u (8 + 3 y) of the result, which must not vanish."""
 import ctypes
 
 import numpy as np
@@ -15,7 +21,8 @@ from paper_1601_04641_gb300 import build
 
 pytestmark = pytest.mark.gpu
 
-SHAPE, D, DT = (20, 12, 40), 1e20, 0.01
+SHAPE, D, DT, U = (20, 12, 40), 1e20, 0.01, 2.0 ** -53
+LD = np.longdouble
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -72,3 +79,26 @@ def test_a_nodes_kick_does_not_depend_on_its_neighbours(form, trap):
         for out in outs:
             assert all(len(np.unique(out[idx == q])) <= 1 for q in range(600))
     assert np.array_equal(outs[0], outs[1])
+
+
+@pytest.mark.parametrize("two_pass", [False, True])
+@pytest.mark.parametrize("form", ["real", "complex"])
+@pytest.mark.parametrize("most", [0.015, 60.0])
+def test_imaginary_time_kick_against_extended_precision(form, most, two_pass):
+    rng = np.random.default_rng(9)
+    amp = np.sqrt(rng.uniform(1e-3, 1.0, SHAPE))
+    psi = amp if form == "real" else amp * np.exp(1j * rng.uniform(-3.0, 3.0, SHAPE))
+    for ax in range(3):
+        np.moveaxis(psi, ax, 0)[[0, -1]] = 0.0
+    g, omega = most / DT, (0.1 / (20 * D)) if most < 1.0 else 0.0
+    out = _kicked(psi, form, g, omega, two_pass)
+    x = [(np.arange(n) - 0.5 * (n - 1)) * D for n in SHAPE]
+    dv = [LD(DT) * LD(0.5) * LD(omega) ** 2 * a.astype(LD) ** 2 for a in x]
+    dv = dv[0][:, None, None] + dv[1][None, :, None] + dv[2][None, None, :]
+    y = LD(DT) * LD(g) * (psi.real.astype(LD) ** 2 + psi.imag.astype(LD) ** 2)
+    assert most > 1.0 or 1e-5 < float(dv.max()) < 0.02
+    exact = psi.astype(LD if form == "real" else np.clongdouble) * np.exp(-(dv + y))
+    bound = U * (1.0 + 8.0 * (dv + y) if most < 1.0 else 8.0 + 3.0 * y)
+    for part in ("real", "imag"):
+        e, o = _interior(getattr(exact, part)), _interior(getattr(out, part))
+        assert np.all(np.abs(o - e) <= _interior(bound) * np.abs(e))
