@@ -543,7 +543,7 @@ gp_status run_stage(gp_handle h, int stage, bool realtime) {
         blocks_for(a.n_lines, pcr.tl) <= h->partial_cap) {
         pcr.levels = at.pcr_levels;
         pcr.lv = h->d_coef + at.off_pcr;
-        pcr.im1 = h->d_coef + at.off_pcr_inv;
+        pcr.inv = h->d_coef + at.off_pcr_inv;
         GP_CK(h, launch_sweep_pcr(L.form, L.kind, a, pcr, h->stream));
     } else {
         GP_CK(h, launch_sweep(L, a, h->stream));

@@ -461,7 +461,7 @@ void append_radial(gp_axial a, int mode, std::vector<char> &host) {
 }
 
 // FP64 tables of the cyclic-reduction form of a mode: the radial matrix's
-// reduction and its right-hand side's coefficients.
+// reduction and its right-hand side's coefficients (doubled, gp_pcr.cuh).
 void append_radial_pcr(gp_axial a, int mode, std::vector<char> &host) {
     using Z = std::complex<double>;
     const int n = a->nx - 2;
@@ -480,7 +480,7 @@ void append_radial_pcr(gp_axial a, int mode, std::vector<char> &host) {
     host.resize(align_up(off + 2 * n * esz, 256), 0);
     for (int t = 0; t < n; ++t)
         for (int q = 0; q < 2; ++q) {
-            const Z v = q ? C[t] : A[t];
+            const Z v = 2.0 * (q ? C[t] : A[t]);
             const double d[2] = {v.real(), v.imag()};
             std::memcpy(host.data() + off + (2 * t + q) * esz, d, esz);
         }
@@ -612,7 +612,7 @@ gp_status run_step(gp_axial a, bool realtime) {
         p.levels = a->rad_levels[mode];
         p.tl = tlr;
         p.lv = a->d_tab + a->rad_pcr[mode][0];
-        p.im1 = a->d_tab + a->rad_pcr[mode][1];
+        p.inv = a->d_tab + a->rad_pcr[mode][1];
         p.rhs = a->d_tab + a->rad_pcr[mode][2];
         AX_CK(a, launch_sweep_pcr(L.form, K_X, x, p, a->stream));
     } else {
@@ -632,7 +632,7 @@ gp_status run_step(gp_axial a, bool realtime) {
         p.levels = zt.pcr_levels;
         p.tl = tlz;
         p.lv = a->d_tab + zt.off_pcr;
-        p.im1 = a->d_tab + zt.off_pcr_inv;
+        p.inv = a->d_tab + zt.off_pcr_inv;
         p.line_w = reinterpret_cast<const double *>(a->d_tab + a->line_w);
         AX_CK(a, launch_sweep_pcr(L.form, K_Z, z, p, a->stream));
         a->cur ^= 1;

@@ -43,8 +43,7 @@ void put_real(char *dst, double v, bool f32) {
 namespace {
 
 // The reduction's tables of the matrix (-a, 1 + e, -c), e the diagonal's
-// excess over one (kept apart from the one, so that 1 / D - 1 keeps its
-// relative accuracy).
+// excess over one (kept apart from the one while the levels change it).
 template <class Z>
 int append_pcr_t(std::vector<char> &host, std::vector<Z> a, std::vector<Z> e, std::vector<Z> c, size_t *off_lv,
                  size_t *off_inv) {
@@ -74,7 +73,6 @@ int append_pcr_t(std::vector<char> &host, std::vector<Z> a, std::vector<Z> e, st
         e.swap(e2);
         c.swap(c2);
     }
-    for (int t = 0; t < n; ++t) inv[t] = -e[t] * inv[t];  // 1 / (1 + e) - 1
     *off_lv = align_up(host.size(), 256);
     *off_inv = align_up(*off_lv + lv.size() * sizeof(Z), 256);
     host.resize(align_up(*off_inv + n * sizeof(Z), 256), 0);

@@ -91,13 +91,13 @@ struct PcrArgs {
     int levels;                    // reduction levels (distances 1, 2, 4, ...)
     int tl;                        // lines per block
     const void *lv;                // [levels][n][2]: A_l[t], C_l[t]
-    const void *im1;               // [n]: 1 / D[t] - 1 after the last level
-    const void *rhs = nullptr;     // [n][2]: A[t], C[t] of the right-hand side (radial lines), null: constant kappa
+    const void *inv;               // [n]: 1 / D[t] after the last level
+    const void *rhs = nullptr;     // [n][2]: 2 A[t], 2 C[t] of the right-hand side (radial lines), null: constant kappa
     bool dependent = false;        // launched as a programmatic dependent (not into graph captures)
     const double *line_w = nullptr;  // z sweep: weight of each line's |phi|^2 in the norm, null: one
 };
 constexpr int kPcrMaxLevels = 10;
-constexpr double kPcrLeft = 0x1p-55;  // coupling left after the last level: a quarter of the unit roundoff
+constexpr double kPcrLeft = 0x1p-55;  // coupling left after the last level: a quarter of the change's unit roundoff
 constexpr size_t kPcrSmem = 100 * 1024;  // most shared memory of a block: two blocks per SM
 constexpr long long kPcrItems = 8 * 1024;  // most (node, line) pairs of a block: 8 per thread
 // Two buffers of the lines' values, the tables (room for the radial form's

@@ -10,17 +10,26 @@
 // the right-hand side and each reduction level run over all (node, line)
 // pairs, with one barrier between them.
 //
-// Cyclic reduction on the CN matrix (-a, D, -c): level l (distance d = 2^l)
-// eliminates the neighbours at distance d,
-//     R[t] <- R[t] + A_l[t] R[t-d] + C_l[t] R[t+d],
-// with A_l, C_l (and the final 1/D - 1) precomputed per node on the host.  The coupling that is left after level l is about
-// |cp|^(2^(l+1)) of the diagonal (cp the Thomas multiplier), so the levels stop
-// when it is below 2^-55 of it, a quarter of the unit roundoff: 4 levels at
-// c = 0.025 (dt = 0.1 d^2), 3 at c = 0.005i, whatever the length of the line.
-// The tables carry the ends of the line (zero beyond them), so every length
-// is served.  Real coefficients cost 3 + 2 levels + 1 operations per
-// component and node against 6 for Thomas: the host takes this form where
-// its better balance outweighs that (choose_pcr).
+// A sweep is solved for the change d = phi - p it makes to the kicked values p:
+// (1 + K) phi = (1 - K) p is (1 + K) d = -2 K p, the same matrix.  Every
+// rounding and the truncation below are then relative to the change, and the
+// one rounding at the size of the field is that of phi = p + d; reducing phi
+// itself rounded each node twice a level at the size of the field and was 1.4
+// to 3 times as far from extended-precision sweeps as the two-pass solve
+// (48x56x40 real, 10 steps: 2.9e-15 of max|psi| against 1.0e-15).
+//
+// Cyclic reduction on the CN matrix (-a, D, -c): level l (distance e = 2^l)
+// eliminates the neighbours at distance e,
+//     R[t] <- R[t] + A_l[t] R[t-e] + C_l[t] R[t+e],
+// with A_l, C_l (and the final 1/D) precomputed per node on the host.  The
+// coupling that is left after level l is about |cp|^(2^(l+1)) of the diagonal
+// (cp the Thomas multiplier), so the levels stop when it is below 2^-55 of it,
+// a quarter of the unit roundoff of the change: 4 levels at c = 0.025
+// (dt = 0.1 d^2), 3 at c = 0.005i, whatever the length of the line.  The tables
+// carry the ends of the line (zero beyond them), so every length is served.
+// Real coefficients cost 3 + 2 levels + 1 operations per component and node
+// against 6 for Thomas: the host takes this form where its better balance
+// outweighs that (choose_pcr).
 #pragma once
 
 #include "gp_async.cuh"
@@ -35,6 +44,19 @@ __device__ __forceinline__ cx<double> pcr_mac(cx<double> acc, double c, cx<doubl
 }
 __device__ __forceinline__ cx<double> pcr_mac(cx<double> acc, cx<double> c, cx<double> v) {
     return cx<double>{fma(c.re, v.re, fma(-c.im, v.im, acc.re)), fma(c.re, v.im, fma(c.im, v.re, acc.im))};
+}
+// 2 c (pm + p1 - 2 p0), c = k / 2 (imaginary time) or i k / 2 (real time)
+template <class F> __device__ __forceinline__ double pcr_rhs(double pm, double p0, double p1, double k) {
+    return k * fma(-2.0, p0, pm + p1);
+}
+template <class F> __device__ __forceinline__ cx<double> pcr_rhs(cx<double> pm, cx<double> p0, cx<double> p1, double k) {
+    const double re = k * fma(-2.0, p0.re, pm.re + p1.re), im = k * fma(-2.0, p0.im, pm.im + p1.im);
+    return real_time<F>() ? cx<double>{-im, re} : cx<double>{re, im};
+}
+__device__ __forceinline__ double pcr_mul(double c, double v) { return c * v; }
+__device__ __forceinline__ cx<double> pcr_mul(double c, cx<double> v) { return cx<double>{c * v.re, c * v.im}; }
+__device__ __forceinline__ cx<double> pcr_mul(cx<double> c, cx<double> v) {
+    return cx<double>{fma(c.re, v.re, -c.im * v.im), fma(c.re, v.im, c.im * v.re)};
 }
 __device__ __forceinline__ double pcr_sub(double a, double b) { return a - b; }
 __device__ __forceinline__ cx<double> pcr_sub(cx<double> a, cx<double> b) { return cx<double>{a.re - b.re, a.im - b.im}; }
@@ -86,8 +108,8 @@ __device__ __forceinline__ void pcr_norm(double v, double *buf, int count, const
 // NS work items per thread (its nodes stay in registers from level to level;
 // shared memory holds what the neighbours read, and the tables).
 // RADIAL: the lines' matrix varies along the line and the right-hand side is
-// p0 + A (pm - p0) + C (p1 - p0) with A, C from p.rhs; the first and the last
-// line (the z boundary) are zero whatever the input holds.
+// 2 A (pm - p0) + 2 C (p1 - p0) with 2 A, 2 C from p.rhs; the first and the
+// last line (the z boundary) are zero whatever the input holds.
 template <class F, int KIND, bool RADIAL, int NS>
 __global__ void __launch_bounds__(1024) lines_pcr_kernel(SweepArgs a, PcrArgs p) {
     using V = typename F::V;
@@ -101,7 +123,7 @@ __global__ void __launch_bounds__(1024) lines_pcr_kernel(SweepArgs a, PcrArgs p)
     V *x = reinterpret_cast<V *>(smem_raw), *y = x + (size_t)p.tl * n;
     C *tab = reinterpret_cast<C *>(y + (size_t)p.tl * n);  // levels, final inverse, radial right-hand side
     const int ntab = 2 * p.levels * n;
-    C *im1 = tab + ntab, *rhs = im1 + n;
+    C *inv = tab + ntab, *rhs = inv + n;
     double *lk = reinterpret_cast<double *>(rhs + (RADIAL ? 2 * n : 0));  // the kick's factor or phase of each line
     const V *in = static_cast<const V *>(a.psi);
     V *out = static_cast<V *>(a.psi_out);
@@ -115,14 +137,14 @@ __global__ void __launch_bounds__(1024) lines_pcr_kernel(SweepArgs a, PcrArgs p)
     // the tables, which no launch writes, while the previous sweep ends
     pdl_trigger();
     for (int q = threadIdx.x; q < ntab; q += T) tab[q] = ldc(static_cast<const C *>(p.lv) + q);
-    for (int q = threadIdx.x; q < n; q += T) im1[q] = ldc(static_cast<const C *>(p.im1) + q);
+    for (int q = threadIdx.x; q < n; q += T) inv[q] = ldc(static_cast<const C *>(p.inv) + q);
     if (RADIAL)
         for (int q = threadIdx.x; q < 2 * n; q += T) rhs[q] = ldc(static_cast<const C *>(p.rhs) + q);
     pdl_wait();
     // item i of the thread: node t of line l of the block (the global
     // accesses of a warp run along the contiguous axis), all ones past the end
     int tt[NS], ll[NS];
-    V v[NS];
+    V p0[NS], v[NS];  // the kicked value, its change
     KickState<double> ks;
     if (KIND == K_X) {
         for (int l = threadIdx.x; l < nl; l += T) {
@@ -136,13 +158,13 @@ __global__ void __launch_bounds__(1024) lines_pcr_kernel(SweepArgs a, PcrArgs p)
         const int s = threadIdx.x + i * T;
         tt[i] = -1;
         ll[i] = 0;
-        v[i] = F::zero();
+        p0[i] = v[i] = F::zero();
         if (s < total) {
             const int m = KIND == K_Z ? n : nl, q = s / m, r = s - q * m;
             tt[i] = KIND == K_Z ? r : q;
             ll[i] = KIND == K_Z ? q : r;
             if (!RADIAL || (L0 + ll[i] > 0 && L0 + ll[i] < lines - 1))
-                v[i] = in[origin(ll[i]) + (long long)(tt[i] + 1) * a.stride];
+                p0[i] = in[origin(ll[i]) + (long long)(tt[i] + 1) * a.stride];
         }
     }
     for (int q = threadIdx.x; q < 2 * nl; q += T)  // the line ends
@@ -153,9 +175,9 @@ __global__ void __launch_bounds__(1024) lines_pcr_kernel(SweepArgs a, PcrArgs p)
         if (tt[i] < 0) continue;
         if (KIND == K_X && (!RADIAL || (L0 + ll[i] > 0 && L0 + ll[i] < lines - 1))) {
             ks.eyz = ks.pyz = lk[ll[i]];
-            v[i] = F::kick(v[i], ks, tt[i] + 1);
+            p0[i] = F::kick(p0[i], ks, tt[i] + 1);
         }
-        x[threadIdx.x + i * T] = v[i];
+        x[threadIdx.x + i * T] = p0[i];
     }
     __syncthreads();
 #pragma unroll
@@ -163,8 +185,8 @@ __global__ void __launch_bounds__(1024) lines_pcr_kernel(SweepArgs a, PcrArgs p)
         const int t = tt[i], s = threadIdx.x + i * T;
         if (t < 0) continue;
         const V pm = t > 0 ? x[s - step] : F::zero(), p1 = t < n - 1 ? x[s + step] : F::zero();
-        if (RADIAL) v[i] = pcr_mac(pcr_mac(v[i], rhs[2 * t], pcr_sub(pm, v[i])), rhs[2 * t + 1], pcr_sub(p1, v[i]));
-        else v[i] = F::rhs(pm, v[i], p1, a.kappa);
+        if (RADIAL) v[i] = pcr_mac(pcr_mul(rhs[2 * t], pcr_sub(pm, p0[i])), rhs[2 * t + 1], pcr_sub(p1, p0[i]));
+        else v[i] = pcr_rhs<F>(pm, p0[i], p1, 2.0 * a.kappa);
         y[s] = v[i];
     }
     for (int lv = 0; lv < p.levels; ++lv) {
@@ -188,7 +210,7 @@ __global__ void __launch_bounds__(1024) lines_pcr_kernel(SweepArgs a, PcrArgs p)
 #pragma unroll
     for (int i = 0; i < NS; ++i) {
         if (tt[i] < 0) continue;
-        const V r = pcr_mac(v[i], im1[tt[i]], v[i]);
+        const V r = pcr_mac(p0[i], inv[tt[i]], v[i]);
         out[origin(ll[i]) + (long long)(tt[i] + 1) * a.stride] = r;
         if (KIND == K_Z && !real_time<F>()) acc = p.line_w ? fma(__ldg(p.line_w + L0 + ll[i]), F::abs2(r), acc) : acc + F::abs2(r);
     }
@@ -220,7 +242,10 @@ inline cudaError_t launch_pcr(const SweepArgs &a, const PcrArgs &p, cudaStream_t
     case 1: return launch_pcr_ns<F, KIND, RADIAL, 1>(a, p, threads, smem, s);
     case 2: return launch_pcr_ns<F, KIND, RADIAL, 2>(a, p, threads, smem, s);
     case 4: return launch_pcr_ns<F, KIND, RADIAL, 4>(a, p, threads, smem, s);
-    default: return launch_pcr_ns<F, KIND, RADIAL, 8>(a, p, threads, smem, s);
+    default:
+        // 16-byte elements have at most 3200 pairs in kPcrSmem
+        if constexpr (sizeof(typename F::V) == 8) return launch_pcr_ns<F, KIND, RADIAL, 8>(a, p, threads, smem, s);
+        else return cudaErrorInvalidValue;
     }
 }
 
