@@ -76,3 +76,77 @@ def test_error_is_no_larger_than_the_two_pass_solves(form, factor):
         errors.append((float(e.max()), float(np.sqrt((e * e).mean()))))
         gp.close()
     assert errors[0][1] <= errors[1][1] and errors[0][0] <= 1.25 * errors[1][0]
+
+
+def _fma(a, b, c):
+    return (a.astype(LD) * b + c).astype(np.float64)
+
+
+def _modelled_real_time(psi, dt):
+    """The two-pass real-time step as its kernel rounds it: a sweep has two roundings a node at the size of the field in the
+    right-hand side and u = r + i k d, two in u / den and ONE in the back substitution, phi = d - (cp phi'), whose product
+    is rounded at its own small size."""
+    re, im = psi.real.copy(), psi.imag.copy()
+    x = [(np.arange(n) - 0.5 * (n - 1)) * H for n in SHAPE]
+    px = [dt * 0.5 * w * w * a * a for w, a in zip(OMEGA, x)]
+    pot, k = px[0][:, None, None] + (px[1][:, None] + px[2][None, :])[None], dt / (4.0 * H * H)
+    kk = np.float64(k)
+
+    def horner(x2, cs):
+        v = np.full_like(x2, cs[0])
+        for c in cs[1:]:
+            v = _fma(x2, v, np.float64(c))
+        return v
+
+    for _ in range(STEPS):
+        th = _fma(np.full_like(re, dt * G), _fma(re, re, im * im), pot)
+        x2 = th * th
+        sn = th * horner(x2, (1.0 / 362880.0, -1.0 / 5040.0, 1.0 / 120.0, -1.0 / 6.0, 1.0))
+        cs = horner(x2, (-1.0 / 3628800.0, 1.0 / 40320.0, -1.0 / 720.0, 1.0 / 24.0, -0.5, 1.0))
+        re, im = _fma(cs, re, sn * im), _fma(cs, im, -sn * re)
+        for ax in range(3):
+            a, b = np.moveaxis(re, ax, 0), np.moveaxis(im, ax, 0)
+            n = a.shape[0] - 2
+            z = np.zeros_like(a[0])
+            cp, d = [], []
+            for t in range(n):
+                e = 2j * k + (1j * k * cp[-1] if t else 0.0)
+                cp.append(-1j * k / (1.0 + e))
+                ip = -e / (1.0 + e)
+                lo, hi = (a[t] if t else z, b[t] if t else z), (a[t + 2] if t < n - 1 else z, b[t + 2] if t < n - 1 else z)
+                dre = _fma(np.full_like(z, -2.0), a[t + 1], lo[0] + hi[0])
+                dim = _fma(np.full_like(z, -2.0), b[t + 1], lo[1] + hi[1])
+                r = _fma(np.full_like(z, -kk), dim, a[t + 1]), _fma(np.full_like(z, kk), dre, b[t + 1])
+                p = d[-1] if t else (z, z)
+                u, v = _fma(np.full_like(z, -kk), p[1], r[0]), _fma(np.full_like(z, kk), p[0], r[1])
+                d.append((_fma(u, ip.real, _fma(-v, ip.imag, u)), _fma(u, ip.imag, _fma(v, ip.real, v))))
+            oa, ob = np.zeros_like(a), np.zeros_like(b)
+            f = d[n - 1]
+            oa[n], ob[n] = f
+            for t in range(n - 2, -1, -1):
+                c = cp[t]
+                f = (d[t][0] - _fma(np.full_like(z, c.real), f[0], -c.imag * f[1]),
+                     d[t][1] - _fma(np.full_like(z, c.real), f[1], c.imag * f[0]))
+                oa[t + 1], ob[t + 1] = f
+            re, im = np.moveaxis(oa, 0, ax), np.moveaxis(ob, 0, ax)
+    return re + 1j * im
+
+
+def test_two_pass_real_time_rounds_as_modelled():
+    """The kernel's error is its model's: 5 roundings a node and sweep.  One more is sqrt(6/5) on a sweep's share, 6 % with
+    the kick's two; two draws of 107 520 errors agree within 1 %."""
+    from paper_1601_04641_gb300.solver import GP
+    f = [np.exp((-0.4 * w + 0.1j) * ((np.arange(n) - 0.5 * (n - 1)) * H - 0.2) ** 2) for n, w in zip(SHAPE, OMEGA)]
+    for v in f:
+        v[0] = v[-1] = 0.0
+    psi = f[0][:, None, None] * f[1][None, :, None] * f[2][None, None, :]
+    psi = np.ascontiguousarray(psi / np.sqrt((np.abs(psi) ** 2).sum() * H ** 3))
+    dt = 0.02 * H * H
+    exact = _reference(psi, dt, False)
+    gp = GP(SHAPE, (H, H, H), dt, OMEGA, G, "f64", "complex")
+    gp.set_window(0)
+    gp.set_psi(psi)
+    gp.step_real(STEPS)
+    rms = [float(np.sqrt((np.abs(f.astype(exact.dtype) - exact) ** 2).mean())) for f in (gp.get_psi(), _modelled_real_time(psi, dt))]
+    gp.close()
+    assert rms[0] <= 1.03 * rms[1]
