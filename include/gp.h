@@ -256,7 +256,8 @@ gp_status gp_sync(gp_handle h);
  * (FP64 arithmetic, not memory, bounds the FP64 forms): two passes with one
  * thread per line, or, on grids with too few lines to fill the GPU that way,
  * cyclic reduction to below a quarter of the unit roundoff.  A window, a
- * segment length or a block size set for an axis keeps the two-pass form. */
+ * segment length, a block size or lines per thread set for an axis keep the
+ * two-pass form. */
 gp_status gp_get_window(gp_handle h, int mode, int window[3]);
 
 /* Override the window of every axis and mode: -1 restores the automatic
@@ -269,8 +270,9 @@ gp_status gp_set_window(gp_handle h, int window);
  * admissible for that axis). */
 gp_status gp_set_axis_window(gp_handle h, int axis, int window);
 
-/* Several adjacent lines per thread on the strided axes (1, the default:
- * the widest group the layout and form allow) or one line per thread (0).
+/* Several adjacent lines per thread on the strided axes (1: the widest group
+ * the layout and form allow) or one line per thread (0).  Until set: 1,
+ * except that FP64 exact solves take one line per thread.
  * A group of g lines needs the axis's line count, and for the y sweep nz, to
  * be a multiple of g.  Pairs serve elements of up to 8 bytes; groups of four
  * serve FP32 real fields with a windowed solve, so that each row a warp
@@ -278,7 +280,7 @@ gp_status gp_set_axis_window(gp_handle h, int axis, int window);
 gp_status gp_set_pair_lines(gp_handle h, int on);
 
 /* The most adjacent lines per thread on one strided axis (axis 0 = x,
- * 1 = y; lines 1, 2 or 4; default 4), within the rules of gp_set_pair_lines.
+ * 1 = y; lines 1, 2 or 4; until set as for gp_set_pair_lines), within its rules.
  * GP_ERR_ARG for another axis or count. */
 gp_status gp_set_lines_per_thread(gp_handle h, int axis, int lines);
 
@@ -341,7 +343,7 @@ gp_status gp_get_segments(gp_handle h, int mode, int seg_len[3], int n_seg[3]);
  * (realtime = 0) or real-time (1) step on this handle's grid under every
  * candidate launch setting -- threads per block (64, 128; for exact solves
  * also 32 and the automatic form), segment length
- * (automatic, 64, 128, 256, whole line) and one or two lines per thread --
+ * (automatic, 64, 128, 256, whole line) and 1, 2 or 4 lines per thread --
  * with CUDA events over `reps` launches after a warm-up, and keep the
  * fastest.  psi is left unchanged (the trials run on a copy).  Choices are
  * cached as text lines "key threads seg pair" in cache_path (NULL: the

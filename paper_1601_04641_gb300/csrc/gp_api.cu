@@ -129,7 +129,8 @@ struct gp_handle_s {
     CUtensorMap zmap[2];
     unsigned int *d_status = nullptr;  // nonzero after a kernel's bounded wait expired
     bool psi_lost = false;             // an expired wait was reported: psi is undefined until set again
-    int max_lpt[2] = {4, 4};   // most adjacent lines per thread on the x and y sweeps (1, 2 or 4)
+    int max_lpt[2] = {0, 0};   // most adjacent lines per thread on the x and y sweeps (1, 2 or 4) set by the
+                               // caller or the autotuner; 0: the form's own (lines_per_thread)
     int seg_override[3] = {0, 0, 0};  // interior nodes per segment, 0 = automatic
     // observables history queued during stepping
     int track_every = 0, track_cap = 0, track_count = 0;
@@ -433,7 +434,7 @@ gp_status check_status(gp_handle h) {
     return GP_OK;
 }
 
-// Adjacent lines per thread on the strided axes, up to max_lpt[ax]: a group
+// Adjacent lines per thread on the strided axes, up to max_lpt[ax] where set: a group
 // of g lines must be adjacent in memory and g-element aligned, i.e. the line
 // count a multiple of g and, for y lines (i, k), nz a multiple of g.  Pairs
 // for elements of 8 bytes or less; groups of four for FP32 real fields with
@@ -441,11 +442,11 @@ gp_status check_status(gp_handle h) {
 int lines_per_thread(gp_handle h, int ax, int window) {
     if (ax == 2 || h->elem > 8) return 1;
     // FP64 exact solves are bound by the FP64 pipe, which a pair does not
-    // relieve: one line a thread, for twice the warps (unless set)
-    if (h->prec == GP_F64 && window == 0 && h->max_lpt[ax] == 4) return 1;
+    // relieve: one line a thread, for twice the warps, unless set
+    const int most = h->max_lpt[ax] ? h->max_lpt[ax] : h->prec == GP_F64 && window == 0 ? 1 : 4;
     auto fits = [&](int g) { return sweep_lines(h, ax) % g == 0 && (ax != 1 || h->n[2] % g == 0); };
-    if (h->max_lpt[ax] >= 4 && (h->elem == 4 || h->elem == 2) && window > 0 && fits(4)) return 4;  // real fields
-    if (h->max_lpt[ax] >= 2 && fits(2)) return 2;
+    if (most >= 4 && (h->elem == 4 || h->elem == 2) && window > 0 && fits(4)) return 4;  // real fields
+    if (most >= 2 && fits(2)) return 2;
     return 1;
 }
 
@@ -534,12 +535,12 @@ gp_status run_stage(gp_handle h, int stage, bool realtime) {
     if (stage == 2 && blocks_for(a.n_lines, zthreads) * (size_t)a.n_seg > h->partial_cap)
         return fail(h, GP_ERR_STATE, "z sweep grid exceeds the partials buffer");
     // FP64 at its automatic settings: by cyclic reduction where the lines are
-    // too few to fill the GPU one thread each (a window, a segment length or
-    // a block size that the caller set keeps the per-thread solve)
+    // too few to fill the GPU one thread each (a window, a segment length, a
+    // block size or lines per thread that the caller set keep the per-thread solve)
     PcrArgs pcr;
     const AxisTables &at = h->tab.ax[mode][ax];
     if (h->prec == GP_F64 && L.window == 0 && h->forced_window < 0 && !h->axis_window[ax] && h->threads[ax] == 0 &&
-        h->seg_override[ax] == 0 && choose_pcr(a.n_lines, a.N - 2, L.form, L.kind, at.pcr_levels, (int)h->elem, &pcr.tl) &&
+        h->seg_override[ax] == 0 && (ax == 2 || h->max_lpt[ax] == 0) && choose_pcr(a.n_lines, a.N - 2, L.form, L.kind, at.pcr_levels, (int)h->elem, &pcr.tl) &&
         blocks_for(a.n_lines, pcr.tl) <= h->partial_cap) {
         pcr.levels = at.pcr_levels;
         pcr.lv = h->d_coef + at.off_pcr;
@@ -1263,7 +1264,7 @@ gp_status gp_pending_scale(gp_handle h, double *scale) {
 namespace {
 
 struct TuneChoice {
-    int threads, seg, lpt;  // lpt: most lines per thread (strided axes)
+    int threads, seg, lpt;  // threads per block and most lines per thread (strided axes), 0: automatic
 };
 
 std::string tune_key(gp_handle h, int realtime, int ax) {
@@ -1330,13 +1331,14 @@ gp_status autotune(gp_handle h, int realtime, int reps, const char *cache_path) 
         const int segs[] = {0, 64, 128, 256, n};
         for (int th : {0, 32, 64, 128})  // 0: the automatic choice
             for (int sg : segs)
-                for (int lp : {4, 2, 1}) {
+                for (int lp : {0, 4, 2, 1}) {
                     if (th <= 32 && h->window[mode][ax] != 0) continue;  // the exact (FP64) form only
-                    if (ax == 2 && lp != 1) continue;  // line groups apply to the strided axes only
+                    // line groups apply to the strided axes only, where the automatic choice is one of both
+                    if (ax == 2 ? lp != 1 : (lp == 0) != (th == 0)) continue;
                     if (ax < 2 && lp == 1 && fp16(h)) continue;  // FP16 storage moves two or four lines
                     if (h->window[mode][ax] == 0 && sg != 0) continue;  // the exact solve has no segments
                     // skip limits that select the same group size as a larger one
-                    if (ax < 2 && lp < 4) {
+                    if (ax < 2 && lp > 0 && lp < 4) {
                         const int keep = h->max_lpt[ax];
                         h->max_lpt[ax] = lp * 2;
                         const int wider = lines_per_thread(h, ax, h->window[mode][ax]);
