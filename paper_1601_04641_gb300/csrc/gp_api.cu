@@ -1267,11 +1267,16 @@ struct TuneChoice {
     int threads, seg, lpt;  // threads per block and most lines per thread (strided axes), 0: automatic
 };
 
+// An FP64 entry is of the levels the cyclic reduction has at this dt (they
+// decide whether it wins), and of the third version: earlier entries always
+// hold a block size, which would keep the reduction from running.
 std::string tune_key(gp_handle h, int realtime, int ax) {
     std::ostringstream k;
     k << h->n[0] << "x" << h->n[1] << "x" << h->n[2] << (h->prec == GP_F32 ? "/f32" : (h->prec == GP_F16 ? "/f16" : "/f64"))
       << (h->field == GP_COMPLEX ? "/c" : "/r") << (realtime ? "/rt" : "/it") << "/w" << h->window[realtime][ax]
-      << "/ax" << ax << "/v2";
+      << "/ax" << ax;
+    if (h->prec == GP_F64) k << "/l" << h->tab.ax[realtime][ax].pcr_levels << "/v3";
+    else k << "/v2";
     return k.str();
 }
 
