@@ -485,14 +485,14 @@ gp_status gp_batch_get_segments(gp_batch b, int i, int seg_len[3], int n_seg[3])
 gp_status gp_batch_set_segments(gp_batch b, int seg_len);
 /* Steps per CUDA graph (default 16; 0 or 1: launch by launch). */
 gp_status gp_batch_set_graph_block(gp_batch b, int steps);
-/* Stream groups of a batched step (1..16, default 2): the active instances
- * are split into groups by the launches they take (line groups on x and y,
- * the z sweep's form; with more than one group asked for, every such kind has
- * at least one) and balanced by sites, and each group's x, y and z sweeps run
- * as one chain of launches on a stream of its own, forked from and joined
- * back into the batch's stream (and captured into its graphs as parallel
- * branches), so launches of different groups overlap.  psi is the same for
- * every setting. */
+/* The most stream groups of a batched step (1..16; until set: two, or one for
+ * every kind of launches where there are more): the active instances are
+ * split into groups by the launches they take (line groups on x and y, the z
+ * sweep's form), or, where there are fewer groups than such kinds, by sites
+ * alone, balanced by sites, and each group's x, y and z sweeps run as one
+ * chain of launches on a stream of its own, forked from and joined back into
+ * the batch's stream (and captured into its graphs as parallel branches), so
+ * launches of different groups overlap.  psi is the same for every setting. */
 gp_status gp_batch_set_streams(gp_batch b, int streams);
 /* z sweep of the instances whose rows fit the TMA form (the rules of
  * gp_set_tma, at the batch's z window; at most 64 instances, the first ones

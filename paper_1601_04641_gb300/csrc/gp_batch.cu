@@ -91,7 +91,7 @@ struct gp_batch_s {
     bool use_tma = true;           // z sweep through TMA for the instances whose rows fit
     int seg_len = 0;               // interior nodes per segment on the strided axes (0: automatic)
     LaunchSet act;                 // the active instances
-    int streams = 2;               // stream groups of a step (1: one chain of launches)
+    int streams = 0;               // most stream groups of a step (1: one chain of launches); 0: not set (stream_groups)
     std::vector<cudaStream_t> gstream;   // the groups' streams (created on first use)
     std::vector<cudaEvent_t> gevent;     // fork event, then one join event per group
     bool dirty = true;
@@ -240,49 +240,13 @@ gp_status build_set(gp_batch b) {
     LaunchSet &S = b->act;
     for (int i = 0; i < b->n; ++i)
         if (b->inst[i].active) S.members.push_back(i);
-    // stream groups: instances that take the same launches (lines per thread
-    // on x and y, the z sweep's form) share groups, so that a group's step is
-    // one launch per sweep wherever there are groups enough; the groups of a
-    // kind (about its share of the sites) are balanced by sites, largest
-    // instance first to the least loaded
-    int ng = std::max(1, std::min(b->streams, (int)S.members.size()));
-    std::vector<std::vector<int>> groups;
-    {
-        std::map<int, std::vector<int>> kinds;
-        std::map<int, size_t> weight;
-        size_t all = 0;
-        for (int i : S.members) {
-            const Inst &I = b->inst[i];
-            const int kind = I.lpt[0] + 4 * I.lpt[1] + (I.ztma ? 16 : 0);
-            kinds[kind].push_back(i);
-            weight[kind] += I.sites;
-            all += I.sites;
-        }
-        // asked for concurrent groups at all, every kind gets one
-        if (b->streams > 1) ng = std::max(ng, (int)kinds.size());
-        groups.resize(ng);
-        std::vector<int> order;
-        for (auto &kv : kinds) order.push_back(kv.first);
-        std::stable_sort(order.begin(), order.end(), [&](int a, int c) { return weight[a] > weight[c]; });
-        std::vector<size_t> load(ng, 0);
-        int used = 0;
-        for (size_t q = 0; q < order.size(); ++q) {
-            const int left = (int)(order.size() - q) - 1;  // kinds still to come keep a group each, while there are any
-            const int want = (int)((double)ng * (double)weight[order[q]] / (double)all + 0.5);
-            const int take = std::max(0, std::min(std::max(1, q + 1 == order.size() ? ng - used : want), ng - used - left));
-            std::vector<int> &v = kinds[order[q]];
-            std::stable_sort(v.begin(), v.end(), [&](int a, int c) { return b->inst[a].sites > b->inst[c].sites; });
-            const int g0 = take > 0 ? used : 0, g1 = take > 0 ? used + take : std::max(1, used);
-            for (int i : v) {
-                const int gi = (int)(std::min_element(load.begin() + g0, load.begin() + g1) - load.begin());
-                groups[gi].push_back(i);
-                load[gi] += b->inst[i].sites;
-            }
-            used += take;
-        }
-        groups.erase(std::remove_if(groups.begin(), groups.end(), [](const std::vector<int> &g) { return g.empty(); }),
-                     groups.end());
+    std::vector<StreamItem> items;
+    for (int i : S.members) {
+        const Inst &I = b->inst[i];
+        items.push_back({i, I.lpt[0] + 4 * I.lpt[1] + (I.ztma ? 16 : 0), I.sites});
     }
+    const std::vector<std::vector<int>> groups = stream_groups(items, b->streams);
+    const int ng = (int)groups.size();
     S.sets.assign(groups.size(), SweepSet());
     for (size_t gs = 0; gs < groups.size(); ++gs) {
         SweepSet &T = S.sets[gs];

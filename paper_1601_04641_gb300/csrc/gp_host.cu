@@ -6,6 +6,7 @@
 #include <cmath>
 #include <complex>
 #include <cstring>
+#include <map>
 
 namespace gpcn {
 
@@ -241,6 +242,52 @@ int default_window(const AxisTables &t, bool f32) {
     // bytes) is faster there.  FP32 is bandwidth-bound and takes the
     // windowed single-pass solve.
     return f32 ? t.min_window : 0;
+}
+
+// Items of one kind share groups, so that a group's step is one launch per
+// sweep (64 uneven complex64 condensates in two mixed groups: 254 us a step;
+// by kind 230); a kind's groups, about its share of the sites, are balanced by
+// sites, the largest item first to the least loaded.  Where fewer groups are
+// asked for than there are kinds, kinds have to mix, and the groups are
+// balanced by sites alone.
+std::vector<std::vector<int>> stream_groups(std::vector<StreamItem> items, int asked) {
+    std::stable_sort(items.begin(), items.end(), [](const StreamItem &a, const StreamItem &b) { return a.sites > b.sites; });
+    std::map<int, std::vector<StreamItem>> kinds;
+    std::map<int, double> weight;
+    double all = 0.0;
+    for (const StreamItem &it : items) {
+        kinds[it.kind].push_back(it);
+        weight[it.kind] += (double)it.sites;
+        all += (double)it.sites;
+    }
+    int ng = std::max(1, std::min(asked > 0 ? asked : 2, (int)items.size()));
+    if (asked == 0) ng = std::max(ng, (int)kinds.size());
+    std::vector<std::vector<int>> groups(ng);
+    std::vector<size_t> load(ng, 0);
+    auto fill = [&](const std::vector<StreamItem> &v, int g0, int g1) {
+        for (const StreamItem &it : v) {
+            const int g = (int)(std::min_element(load.begin() + g0, load.begin() + g1) - load.begin());
+            groups[g].push_back(it.id);
+            load[g] += it.sites;
+        }
+    };
+    if (ng < (int)kinds.size()) {
+        fill(items, 0, ng);
+    } else {
+        std::vector<int> order;
+        for (auto &kv : kinds) order.push_back(kv.first);
+        std::stable_sort(order.begin(), order.end(), [&](int a, int c) { return weight[a] > weight[c]; });
+        int used = 0;
+        for (size_t q = 0; q < order.size(); ++q) {
+            const int left = (int)(order.size() - q) - 1;  // kinds still to come keep a group each
+            const int want = left ? std::max(1, (int)(ng * weight[order[q]] / all + 0.5)) : ng - used;
+            const int take = std::min(want, ng - used - left);
+            fill(kinds[order[q]], used, used + take);
+            used += take;
+        }
+    }
+    groups.erase(std::remove_if(groups.begin(), groups.end(), [](const std::vector<int> &g) { return g.empty(); }), groups.end());
+    return groups;
 }
 
 long long axis_lines(const Geometry &G, int ax) {

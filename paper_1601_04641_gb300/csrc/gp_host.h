@@ -56,6 +56,15 @@ int append_pcr(std::vector<char> &host, const std::vector<std::complex<double>> 
 // cyclic reduction than by the exact two-pass solve, and its lines per block.
 bool choose_pcr(long long lines, int n, Form form, Kind kind, int levels, int elem_bytes, int *tl);
 
+// Stream groups of a batched step: item ids per group, none empty.  A kind is
+// a set of launches (lines per thread on x and y, the z sweep's form);
+// `asked` groups at most, 0: automatic, two or one per kind.
+struct StreamItem {
+    int id, kind;
+    size_t sites;
+};
+std::vector<std::vector<int>> stream_groups(std::vector<StreamItem> items, int asked);
+
 // Default window of an axis: the smallest admissible one in FP32 (bandwidth
 // bound), the exact two-pass solve (0) in FP64 (ALU bound).
 int default_window(const AxisTables &t, bool f32);

@@ -1,5 +1,6 @@
 // Asks libgpcn.so's host side (no GPU) what it would do; see test_host_rules.py.
 //   optin                             the calls a kernel's opt-in makes: per device, per growth, on failure, from threads
+//   streams ASKED KIND SITES ...      the groups of a batched step, a line of item numbers each
 //   tables NX NY NZ MODES DT DT ...   tables built for each dt in turn into one Tables, against fresh ones: 1 where equal
 #include "gp_host.h"
 #include "gp_optin.h"
@@ -58,6 +59,16 @@ static int optin() {
 
 int main(int argc, char **argv) {
     if (argc > 1 && !std::strcmp(argv[1], "optin")) return optin();
+    if (argc > 4 && !std::strcmp(argv[1], "streams")) {
+        std::vector<StreamItem> items;
+        for (int q = 3; q + 1 < argc; q += 2)
+            items.push_back({(int)items.size(), std::atoi(argv[q]), (size_t)std::atoll(argv[q + 1])});
+        for (const auto &g : stream_groups(items, std::atoi(argv[2]))) {
+            for (int i : g) std::printf("%d ", i);
+            std::printf("\n");
+        }
+        return 0;
+    }
     if (argc > 6 && !std::strcmp(argv[1], "tables")) {
         Geometry G;
         for (int q = 0; q < 3; ++q) {

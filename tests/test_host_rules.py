@@ -1,6 +1,7 @@
 """The host rules that choose kernels and lay out their tables, asked of
 libgpcn.so itself through a small C++ client (no GPU)."""
 import os
+import random
 import re
 import subprocess
 
@@ -51,3 +52,24 @@ def test_no_launcher_keeps_a_process_wide_opt_in():
     for name in sorted(os.listdir(build.CSRC)):
         src = open(os.path.join(build.CSRC, name)).read()
         assert not re.search(r"static\s+(bool|int)\s+attr\b", src), name
+
+
+@pytest.mark.parametrize("asked", [0, 1, 2, 3, 5, 16])
+@pytest.mark.parametrize("kinds", [1, 2, 4, 8])
+def test_stream_groups_are_no_more_than_asked_for(probe, asked, kinds):
+    """Every instance in one group; at most as many groups as set, where not set two or one per kind; groups of one kind
+    wherever there are enough of them; balanced by sites within the largest instance."""
+    rng = random.Random(7)
+    items = [(rng.randrange(kinds) if q >= kinds else q, rng.randrange(1000, 50000)) for q in range(24)]
+    groups = [[int(v) for v in g] for g in probe("streams", asked, *[v for it in items for v in it])]
+    assert sorted(i for g in groups for i in g) == list(range(24))
+    most = asked or max(2, kinds)
+    assert len(groups) == min(most, 24)
+    if most >= kinds:
+        assert all(len({items[i][0] for i in g}) == 1 for g in groups)
+        shared = [[g for g in groups if items[g[0]][0] == k] for k in range(kinds)]
+    else:
+        shared = [groups]
+    for gs in shared:
+        load = [sum(items[i][1] for i in g) for g in gs]
+        assert max(load) - min(load) <= max(items[i][1] for g in gs for i in g)
