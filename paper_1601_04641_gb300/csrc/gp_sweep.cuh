@@ -1372,20 +1372,22 @@ __device__ __forceinline__ double lines_body(const SweepArgs &a, unsigned bx, un
     return acc.value();
 }
 
-// One thread per (line, segment), or per (pair of adjacent lines, segment)
-// when LPT = 2; blockIdx.y is the segment.  Window 0 selects the exact
-// two-pass form over whole lines with direct access.
 // Blocks of 64 threads per SM that the compiler leaves registers for: eight
 // (128 registers, no spills) for single FP32 lines of windows 4 and 8, whose
 // rings leave room for as many (241x201x161 complex64 imaginary time 1.29 ->
-// 1.17 ms per 10 steps).  Line groups keep theirs: held to 128, complex64 real
-// time gained 1 % on 480x400x320 and lost 4 % on 200x160x120, where two blocks
-// an SM are all there are; wider windows spill.
+// 1.17 ms per 10 steps), and of window 16 for real fields (left to itself the
+// compiler takes 166 for the batched x sweep, six blocks an SM: 64 real
+// condensates at window 16 219 us a step, held to 128 206).  Line groups keep
+// theirs: held to 128, complex64 real time gained 1 % on 480x400x320 and lost
+// 4 % on 200x160x120, where two blocks an SM are all there are; complex lines of
+// window 16 spill.
 template <class F, int W, int LPT> __host__ __device__ constexpr int lines_min_blocks() {
-    return sizeof(typename F::Real) == 4 && (W == 4 || W == 8) && LPT == 1 ? 8 : 1;
+    return sizeof(typename F::Real) == 4 && (W == 4 || W == 8 || (W == 16 && sizeof(typename F::V) == 4)) && LPT == 1 ? 8 : 1;
 }
 
-// TB: threads per block, 0 for any.
+// One thread per (line, segment), or per (group of LPT adjacent lines,
+// segment); blockIdx.y is the segment.  Window 0 selects the exact two-pass
+// form over whole lines with direct access.  TB: threads per block, 0 for any.
 template <class F, typename R, int W, int KIND, int LPT, int TB>
 __global__ void __launch_bounds__(TB > 0 ? TB : 256, TB > 0 ? lines_min_blocks<F, W, LPT>() : 1) sweep_lines_kernel(SweepArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
