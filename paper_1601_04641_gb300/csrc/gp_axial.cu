@@ -602,7 +602,13 @@ gp_status run_step(gp_axial a, bool realtime) {
     SweepLaunch L;
     L.prec = f32_of(a) ? P_F32 : P_F64;
     L.form = realtime ? F_REALTIME : (a->field == GP_REAL ? F_IMAG_REAL : F_IMAG_CPLX);
-    const int tlr = pcr_lines(a, L.form, K_X, a->nz, a->nx - 2, a->rad_levels[mode]);
+    // in imaginary time the reduction's kick multiplies by deviations from one,
+    // which leave nothing of a trap factor below the unit roundoff (e^-37); up
+    // to e^-30 a product of them stays apart from zero, and beyond that the
+    // radial kernels below take the exponential of the whole exponent
+    const double rmax = (a->nx - 2.5) * a->drho, zmax = 0.5 * (a->nz - 3) * a->dz;
+    const double trap = 0.5 * a->dt * (a->gamma * a->gamma * rmax * rmax + a->lambda * a->lambda * zmax * zmax);
+    const int tlr = realtime || trap <= 30.0 ? pcr_lines(a, L.form, K_X, a->nz, a->nx - 2, a->rad_levels[mode]) : 0;
     if (tlr > 0) {
         SweepArgs x = sweep_args(G, 0, realtime, r.in, r.out, a->d_tab, a->T, 0, 1, r.scale, nullptr, nullptr, nullptr, nullptr);
         if (realtime) x.phase_ex = a->d_tab + a->rad_phase;
