@@ -722,7 +722,11 @@ gp_status gp_axial_create(gp_axial *out, int nx, int nz, double drho, double dz,
     append_tables(geom_of(a), prec == GP_F32, modes_of(a), host, a->T, kPcrAll);
     for (int mode = 0; mode < modes_of(a); ++mode) append_radial(a, mode, host);
     if (prec == GP_F64) {
-        for (int mode = 0; mode < modes_of(a); ++mode) append_radial_pcr(a, mode, host);
+        // only where one line at least fits a block (with the fewest levels: a
+        // line of 10^6 nodes would get 144 MB of tables that nothing reads)
+        for (int mode = 0; mode < modes_of(a); ++mode)
+            if (pcr_lines(a, mode == 1 ? F_REALTIME : field == GP_REAL ? F_IMAG_REAL : F_IMAG_CPLX, K_X, nz, nx - 2, 1) > 0)
+                append_radial_pcr(a, mode, host);
         append_radial_nodes(a, host);
     }
     a->part_cap = std::max((size_t)kRedBlocks * 6, ((size_t)nx + 31) / 32 * (size_t)(nz > 2 ? nz - 2 : 1) + 64);

@@ -34,3 +34,19 @@ def test_trap_factors_below_the_roundoff(field, drho, dt):
     oracle.axial_step(ref, drho, dz, dt, gamma, lam, g, False, 2)
     assert abs(obs["norm"] - 1.0) <= 1e-12
     assert np.max(np.abs(got - ref)) <= 6e-14 * np.max(np.abs(ref))
+
+
+def test_a_long_radial_line_gets_no_reduction_tables():
+    """2e6 radial nodes: two fields (96 MB), the radial two-pass tables (128), the Cartesian ones (80) and the nodes' (48);
+    the reduction's, for lines that no block can hold, would add at least 144."""
+    import torch
+    from paper_1601_04641_gb300.solver import AxialGP
+    torch.cuda.empty_cache()
+    free = torch.cuda.mem_get_info()[0]
+    a = AxialGP(2000000, 3, 0.5, 0.5, 1e-3, 1e-9, 1.0, 1.0, "f64", "real")
+    used = free - torch.cuda.mem_get_info()[0]
+    a.init_gaussian()
+    a.step_imag(1)
+    assert abs(a.observables()["norm"] - 1.0) <= 1e-10
+    a.close()
+    assert used <= 400e6
