@@ -107,32 +107,44 @@ static int pcr_levels(std::complex<double> c) {
     return 0;
 }
 
-// Both forms are bound by the FP64 pipe: 64 clocks per warp instruction and
-// SM sub-partition (152 SMs of four).  Thomas: a warp holds 32 lines for all
-// of its n nodes, so the busiest sub-partition has ceil(warps / 608) of them;
-// cyclic reduction spreads the nodes of a block's lines over the SM's four.
-// Operations per node and component as the kernels' forms have them (kick:
-// 12, 14, 16; norm 1 or 2).  64x48x40 real: x 62 x 18 against 8 x 24.
+// Both forms are bound by the FP64 pipe, in units of 64 clocks: what one warp
+// instruction takes on an SM of up to four warps; with more the pipe is shared,
+// w / 4 each.  Thomas: a warp holds 32 lines for all of its n nodes (blocks of
+// one warp on x and y, of two on z).  Cyclic reduction: the nodes of a block's
+// lines are spread over the SM's four sub-partitions, one block after the
+// other.  Operations per node and component as the kernels' forms have them
+// (kick 15, 18, 19; the reduction's real-time kick multiplies by the pending
+// factor, two more; norm, imaginary time only, 1 or 2).
+// Timed on both sides, us a step of three sweeps with one axis changed from
+// Thomas to the reduction (gain), and the two counts:
+//   64x48x40 real x            41.7   1302 / 189    96x96x96 real y    6.3    564 / 540
+//   96x96x96 complex dt y      7.1   1128 / 1104   160x128x96 real x  12.7   3318 / 2754
+//   160x128x96 real z         -5.7    987 / 1300   60x120x180 real x  -2.1   1523 / 1755
+//   90x157x150 real x        -13.2   2310 / 2916   128x128x128 real x -5.9   2646 / 2916
+//   112x112x112 real time x   -1.9   4070 / 4125   30x150x150 real x  -2.1    735 / 891
+// (counting each started wave of 608 Thomas warps as a whole one took the
+// reduction on 60x120x180, 90x157x150 and 160x128x96 z, up to 10 % of a step slower).
 bool choose_pcr(long long lines, int n, Form form, Kind kind, int levels, int elem_bytes, int *tl) {
     if (levels < 1 || n < 1 || lines < 1 || lines > 0x7fffffffLL) return false;
     constexpr long long kSms = 152;
-    const int extra = kind == K_X ? (form == F_IMAG_REAL ? 12 : form == F_IMAG_CPLX ? 14 : 16)
-                                  : kind == K_Z ? (form == F_IMAG_REAL ? 1 : 2) : 0;
-    const int thomas_ops = (form == F_IMAG_REAL ? 6 : form == F_IMAG_CPLX ? 12 : 16) + extra;
-    const int pcr_ops = (form == F_IMAG_REAL ? 4 + 2 * levels : form == F_IMAG_CPLX ? 8 + 4 * levels : 10 + 8 * levels) + extra;
+    const bool rt = form == F_REALTIME, re = form == F_IMAG_REAL;
+    const int extra = kind == K_X ? (re ? 15 : rt ? 19 : 18) : kind == K_Z && !rt ? (re ? 1 : 2) : 0;
+    const int thomas_ops = (re ? 6 : rt ? 18 : 12) + extra;
+    const int pcr_ops = (re ? 4 + 2 * levels : rt ? 10 + 8 * levels : 8 + 4 * levels) + extra + (kind == K_X && rt ? 2 : 0);
     auto up = [](long long a, long long b) { return (a + b - 1) / b; };
-    const long long thomas = up(up(lines, 32), 4 * kSms) * n * thomas_ops;
+    const long long warps = kind == K_Z ? 2 * up(up(lines, 64), kSms) : up(up(lines, 32), kSms);  // of an SM, at most
+    const long long thomas4 = std::max(4LL, warps) * n * thomas_ops;  // four times the units
     long long best = -1;
     for (int per_sm = 1; per_sm <= 16; ++per_sm) {
         const long long t = up(lines, kSms * per_sm);
-        if (t * n > kPcrItems || pcr_smem(elem_bytes, form == F_REALTIME ? 16 : 8, levels, (int)t, n + 2) > kPcrSmem) continue;
+        if (t * n > kPcrItems || pcr_smem(elem_bytes, rt ? 16 : 8, levels, (int)t, n + 2) > kPcrSmem) continue;
         const long long cost = up(up(lines, t), kSms) * up(t * n, 128) * pcr_ops;
         if (best < 0 || cost < best) {
             best = cost;
             *tl = (int)t;
         }
     }
-    return best >= 0 && best < thomas;
+    return best >= 0 && 4 * best < thomas4;
 }
 
 void append_tables(const Geometry &G, bool f32, int modes, std::vector<char> &host, Tables &T, PcrTables pcr) {

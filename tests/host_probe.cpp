@@ -1,6 +1,7 @@
 // Asks libgpcn.so's host side (no GPU) what it would do; see test_host_rules.py.
 //   optin                             the calls a kernel's opt-in makes: per device, per growth, on failure, from threads
 //   streams ASKED KIND SITES ...      the groups of a batched step, a line of item numbers each
+//   choose LINES N FORM KIND LEVELS ELEM   whether the cyclic reduction is chosen, and its lines per block
 //   tables NX NY NZ MODES DT DT ...   tables built for each dt in turn into one Tables, against fresh ones: 1 where equal
 #include "gp_host.h"
 #include "gp_optin.h"
@@ -59,6 +60,13 @@ static int optin() {
 
 int main(int argc, char **argv) {
     if (argc > 1 && !std::strcmp(argv[1], "optin")) return optin();
+    if (argc == 8 && !std::strcmp(argv[1], "choose")) {
+        int tl = 0;
+        const bool yes = choose_pcr(std::atoll(argv[2]), std::atoi(argv[3]), (Form)std::atoi(argv[4]), (Kind)std::atoi(argv[5]),
+                                    std::atoi(argv[6]), std::atoi(argv[7]), &tl);
+        std::printf("%d %d\n", yes ? 1 : 0, tl);
+        return 0;
+    }
     if (argc > 4 && !std::strcmp(argv[1], "streams")) {
         std::vector<StreamItem> items;
         for (int q = 3; q + 1 < argc; q += 2)

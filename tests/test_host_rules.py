@@ -73,3 +73,32 @@ def test_stream_groups_are_no_more_than_asked_for(probe, asked, kinds):
     for gs in shared:
         load = [sum(items[i][1] for i in g) for g in gs]
         assert max(load) - min(load) <= max(items[i][1] for g in gs for i in g)
+
+
+# grid, form (0 real, 1 complex, 2 real time), levels, axis, us a step gained by the reduction on that axis (measured)
+CROSSOVER = [
+    ((64, 48, 40), 0, 4, 0, 41.7), ((80, 80, 80), 0, 4, 1, 10.4), ((80, 80, 80), 2, 4, 0, 45.5), ((96, 96, 96), 0, 4, 1, 6.3),
+    ((96, 96, 96), 0, 4, 2, 7.3), ((96, 96, 96), 1, 4, 1, 7.1), ((112, 112, 112), 0, 4, 0, 8.5), ((160, 128, 96), 0, 4, 0, 12.7),
+    ((40, 200, 300), 2, 3, 2, 41.7), ((150, 60, 250), 2, 3, 2, 30.8),
+    ((160, 128, 96), 0, 4, 2, -5.7), ((160, 128, 96), 1, 4, 2, -19.6), ((60, 120, 180), 1, 4, 0, -7.2),
+    ((60, 120, 180), 0, 5, 0, -6.3), ((90, 157, 150), 0, 4, 0, -13.2), ((90, 157, 150), 2, 3, 0, -29.1),
+    ((128, 128, 128), 0, 4, 0, -5.9), ((200, 160, 120), 0, 4, 1, -38.4), ((30, 150, 150), 1, 4, 0, -7.3),
+]
+
+
+@pytest.mark.parametrize("shape,form,levels,axis,gain", CROSSOVER)
+def test_the_choice_of_the_reduction_follows_the_measurements(probe, shape, form, levels, axis, gain):
+    lines = shape[0] * shape[1] * shape[2] // shape[axis]
+    (chosen, tl), = probe("choose", lines, shape[axis] - 2, form, axis, levels, 8 if form == 0 else 16)
+    assert bool(chosen) == (gain > 0)
+
+
+@pytest.mark.parametrize("form,elem", [(0, 8), (1, 16), (2, 16)])
+def test_a_blocks_lines_fit_its_threads_and_shared_memory(probe, form, elem):
+    for shape in ((64, 48, 40), (100, 90, 80), (90, 157, 150), (20, 300, 300), (400, 20, 30), (3, 3, 3)):
+        for axis in range(3):
+            n, lines = shape[axis] - 2, shape[0] * shape[1] * shape[2] // shape[axis]
+            for levels in range(1, 11):
+                _, tl = probe("choose", lines, n, form, axis, levels, elem)[0]
+                assert tl * n <= (8192 if elem == 8 else 4096)
+                assert tl == 0 or tl * (2 * n * elem + 8) + n * (2 * levels + 3) * (16 if form == 2 else 8) <= 100 * 1024
