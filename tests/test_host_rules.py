@@ -102,3 +102,28 @@ def test_a_blocks_lines_fit_its_threads_and_shared_memory(probe, form, elem):
                 _, tl = probe("choose", lines, n, form, axis, levels, elem)[0]
                 assert tl * n <= (8192 if elem == 8 else 4096)
                 assert tl == 0 or tl * (2 * n * elem + 8) + n * (2 * levels + 3) * (16 if form == 2 else 8) <= 100 * 1024
+
+
+def test_gpu_block_cases_reach_every_form(probe):
+    """The grids of test_gpu_pcr_blocks.py take the reduction with 1, 2, 4 and (real fields) 8 pairs a thread, with more than
+    48 KB of shared memory, and with 3 to 10 levels."""
+    from tests import test_gpu_pcr_blocks as blocks
+    seen, big, levels_seen = set(), False, set()
+    for form, elem in ((0, 8), (1, 16), (2, 16)):
+        for shape in blocks.SHAPES:
+            for factor in blocks.FACTORS:
+                c = factor / 4.0 * (1j if form == 2 else 1.0)
+                b, levels = c / (1.0 + 2.0 * c), 0
+                while levels == 0 or 2.0 * abs(b) > 2.0 ** -55:
+                    b, levels = b * b / (1.0 - 2.0 * b * b), levels + 1
+                if levels > 10:
+                    continue
+                for axis in range(3):
+                    n, lines = shape[axis] - 2, shape[0] * shape[1] * shape[2] // shape[axis]
+                    (chosen, tl), = probe("choose", lines, n, form, axis, levels, elem)
+                    if chosen:
+                        seen.add((form, 1 if tl * n <= 1024 else 2 if tl * n <= 2048 else 4 if tl * n <= 4096 else 8))
+                        big |= tl * 2 * n * elem > 48 * 1024
+                        levels_seen.add(levels)
+    assert seen == {(0, 1), (0, 2), (0, 4), (0, 8), (1, 1), (1, 2), (1, 4), (2, 1), (2, 2), (2, 4)}
+    assert big and levels_seen >= set(range(4, 11)) - {6, 7}
