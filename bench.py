@@ -52,12 +52,12 @@ BATCH_WORKLOADS = {"batch64_c64": "complex", "batch64_real": "real"}
 
 # FP64 arithmetic of the FP64 complex real-time step, counted from the
 # kernels' operations (an FMA is 2 flops, a multiply or add 1): the kick
-# 26 per site (|q|^2 3, phase 3, sin/cos series near zero 14, rotation 6; no
-# scale is pending in real time); each line solve 30 per node (right-hand side 10, forward 12, backward 8),
-# three of them; the observables 29 per site per call.  The FP64 peak is the
+# 32 per site (|q|^2 3, phase 3, sin/cos series 20, rotation 6; no scale is
+# pending in real time); each line solve 30 per node (right-hand side 10,
+# forward 12, backward 8), three of them; the observables 29 per site per call.  The FP64 peak is the
 # profiling recipe's nominal 1.25 TFLOP/s (an FMA-chain probe on this part
 # measured 1.255).
-FP64_FLOPS_STEP_REALTIME = 26 + 3 * 30
+FP64_FLOPS_STEP_REALTIME = 32 + 3 * 30
 FP64_FLOPS_OBSERVABLES = 29
 FP64_PEAK_GFLOPS = 1250.0
 

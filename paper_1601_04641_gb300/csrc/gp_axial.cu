@@ -233,9 +233,9 @@ __global__ void __launch_bounds__(kRadialThreads) axial_radial_smem_kernel(AxArg
 // 6 quantities (or the first alone), added in block order by the last block
 // to finish (deterministic).  One site per thread on a 120x241 grid: the sums
 // are bound by the FP64 pipe, which works at 64 clocks per warp instruction
-// however few lanes are active, so the blocks are many and short.  (One block
-// adding 304 partials with one thread per quantity took 27 us, the sums with
-// a division per site 14 us; now 4 us together.)
+// however few lanes are active, so the blocks are many and short.  (In launch
+// lists: sums with a division per site 14 us and one block that added 304
+// partials with one thread per quantity 27; this kernel 11.)
 constexpr int kRedThreads = 192;  // one warp per quantity in the last block
 constexpr int kRedBlocks = 304;
 

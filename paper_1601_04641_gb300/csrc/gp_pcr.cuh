@@ -1,11 +1,10 @@
 // gp_pcr.cuh -- FP64 line solves by truncated parallel cyclic reduction.
 //
-// The FP64 pipe of this part issues one warp instruction per 64 clock cycles
-// and SM sub-partition (measured: 64.4 with independent operations, 66 in a
-// dependent chain, the same for 1 to 32 active lanes), so an FP64 sweep costs
-// 64 cycles times the warp instructions of its busiest sub-partition and a
-// one-thread-per-line Thomas solve of a small grid leaves most of the 608
-// sub-partitions idle: 64x48x40 has 60 warps of x lines.  Here a block keeps
+// One FP64 warp instruction takes 64 clock cycles on this part (measured: 64.4
+// with independent operations, 66 in a dependent chain, the same for 1 to 32
+// active lanes), up to four warps of an SM side by side, more sharing the
+// pipe, and a one-thread-per-line Thomas solve of a small grid leaves most of
+// the SMs' room for 608 idle: 64x48x40 has 60 warps of x lines.  Here a block keeps
 // `tl` whole lines in shared memory and every node is a work item: the kick,
 // the right-hand side and each reduction level run over all (node, line)
 // pairs, with one barrier between them.

@@ -924,14 +924,13 @@ template <typename V> __host__ __device__ constexpr int chunk_len() { return siz
 // readable, two in flight.
 constexpr int kRingChunks = 4;
 
-// Windowed Thomas solve of the interior nodes [tb, te) of a line of n
-// interior unknowns; the coefficient tables hold their last values from
-// tconst on.
-// interior unknowns.  Inputs are read by interior position p (node p+1;
-// positions outside [0, n) read 0) after io.need(p_end) has made the
-// positions [p_end - B, p_end) readable; outputs go through io.put(t0, q, v)
-// (position t0 + q) and io.flush(t0, count).
-// One full chunk: dp[t0+W .. t0+W+B-1] forward, then phi[t0 .. t0+B-1] by
+// Windowed Thomas solve (solve_segment) of the interior nodes [tb, te) of a
+// line of n interior unknowns; the coefficient tables hold their last values
+// from tconst on.  Inputs are read by interior position p (node p+1; positions
+// outside [0, n) read 0) after io.need(p_end) has made the positions
+// [p_end - B, p_end) readable; outputs go through io.put(t0, q, v) (position
+// t0 + q) and io.flush(t0, count).
+// window_chunk, one full chunk: dp[t0+W .. t0+W+B-1] forward, then phi[t0 .. t0+B-1] by
 // the windowed backward sweep.  SETTLED: every coefficient the chunk uses
 // equals the table's last entry (cp and ip reach their fixed point a few
 // nodes into the line and stay there to FP rounding), so they are read once
@@ -1235,9 +1234,9 @@ template <class F, class M, typename R, int KIND> struct DirectIO {
 // (A ring of four chunks from the segment's first position, masked per node,
 // spent 20 integer instructions per site on the complex64 x sweep.)
 // Where that start lies 12 nodes before the segment's first input (chunks of
-// 16, windows 8 and 16), a short line would wait for one more chunk (64 FP32
-// real condensates at window 16: 0.229 -> 0.237 ms a step): those forms keep
-// the ring of four from the first position.
+// 16, windows 8 and 16), aligned lines read one chunk more for nothing: those
+// forms keep the ring of four from the first position (64 FP32 real
+// condensates at window 16: 235.5 us a step so, 236.6 aligned, no difference).
 template <int B, int W> __host__ __device__ constexpr bool column_aligned() {
     return (2 * W + 4 + B - 1) / B * B - (2 * W + 4) <= 4;
 }
