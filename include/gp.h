@@ -161,7 +161,8 @@ gp_status gp_get_psi(gp_handle h, void *psi, int on_device);
 /* Change g (a quench); the CN coefficients do not depend on g. */
 gp_status gp_set_g(gp_handle h, double g);
 
-/* Change dt; rebuilds the CN coefficient tables. */
+/* Change dt; rebuilds the CN coefficient tables (FP64 ones may need more
+ * device memory: GP_ERR_NOMEM leaves the handle at its old dt). */
 gp_status gp_set_dt(gp_handle h, double dt);
 
 /* Queue nsteps imaginary-time steps: kick, x, y and z line solves, then
